@@ -35,15 +35,26 @@ __device__ __forceinline__ M3 m3dag(const M3& a) {
   return r;
 }
 
-// link U_mu at global coordinates x + shift (periodic), from the FP64 copy
-__device__ __forceinline__ M3 link_at(const Geom& g, const double2* U64, const int x[4], int mu, int s0, int s1,
-                                      int d0, int d1) {
-  int y[4];  // selects only, no dynamically indexed writes
+// q - q^+ of the product q = a b in 9 reals: twice the imaginary diagonal,
+// then (re, im) of the elements (0,1), (0,2), (1,2).  The real diagonal is never
+// formed, which leaves 90 of a product's 108 FP64 operations.
+__device__ __forceinline__ void antiherm_product(const M3& a, const M3& b, double t[9]) {
+  const M3 q = m3mul(a, b);
 #pragma unroll
-  for (int d = 0; d < 4; ++d) y[d] = (x[d] + (d == d0 ? s0 : 0) + (d == d1 ? s1 : 0) + g.L[d]) % g.L[d];
-  long long s = internal_index(g, y);
-  int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
-  SU3<double> u = load_link<P64, double>(U64, g.Vb, blk, r, mu);
+  for (int i = 0; i < 3; ++i) t[i] = 2.0 * q.m[i][i].im;
+  int k = 3;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i + 1; j < 3; ++j) {
+      t[k++] = q.m[i][j].re - q.m[j][i].re;
+      t[k++] = q.m[i][j].im + q.m[j][i].im;
+    }
+}
+
+__device__ __forceinline__ M3 link_of(const Geom& g, const double2* U64, long long s, int mu) {
+  const int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
+  const SU3<double> u = load_link<P64, double>(U64, g.Vb, blk, r, mu);
   M3 o;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -52,42 +63,97 @@ __device__ __forceinline__ M3 link_at(const Geom& g, const double2* U64, const i
   return o;
 }
 
-// Fhat_{mu nu}(x) = (Q - Q^+) / 8, Q = sum of the four counter-clockwise leaves at x
-__device__ M3 fhat(const Geom& g, const double2* U64, const int x[4], int mu, int nu) {
-  // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
-  M3 q = m3mul(m3mul(link_at(g, U64, x, mu, 0, 0, mu, nu), link_at(g, U64, x, nu, 1, 0, mu, nu)),
-               m3mul(m3dag(link_at(g, U64, x, mu, 0, 1, mu, nu)), m3dag(link_at(g, U64, x, nu, 0, 0, mu, nu))));
-  // leaf 2: U_nu(x) U_mu(x+nu-mu)^+ U_nu(x-mu)^+ U_mu(x-mu)
-  M3 l = m3mul(m3mul(link_at(g, U64, x, nu, 0, 0, mu, nu), m3dag(link_at(g, U64, x, mu, -1, 1, mu, nu))),
-               m3mul(m3dag(link_at(g, U64, x, nu, -1, 0, mu, nu)), link_at(g, U64, x, mu, -1, 0, mu, nu)));
+// internal index of x + s_mu mu-hat + s_nu nu-hat (periodic; selects only, no
+// dynamically indexed writes)
+__device__ __forceinline__ long long site_at(const Geom& g, const int x[4], int mu, int smu, int nu, int snu) {
+  int y[4];
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int d = 0; d < 4; ++d) y[d] = (x[d] + (d == mu ? smu : 0) + (d == nu ? snu : 0) + g.L[d]) % g.L[d];
+  return internal_index(g, y);
+}
+
+// the j-th of a site's 72 reals in a clover record's memory ([blk][36 double2][Vb]),
+// which the build uses as scratch: a site's reals are its own, so the last pass can
+// turn them into the record in place
+__device__ __forceinline__ double* rec_real(double* rec, const Geom& g, long long s, int j) {
+  const long long blk = s / g.Vb, r = s - blk * g.Vb;
+  return rec + 2 * ((blk * 36 + (j >> 1)) * g.Vb + r) + (j & 1);
+}
+
+// planes 0 .. 5 in the order 01, 23, 02, 13, 03, 12: a launch takes two of them
+__device__ __forceinline__ void plane_dirs(int q, int& mu, int& nu) {
+  mu = (q & 1) == 0 ? 0 : (q == 5 ? 1 : (q == 3 ? 1 : 2));
+  nu = q == 0 ? 1 : (q == 1 ? 3 : (q == 2 ? 2 : (q == 3 ? 3 : (q == 4 ? 3 : 2))));
+}
+
+// The four leaves of one plaquette (x; mu < nu), one thread each, for the plane
+// q0 + blockIdx.y.  A leaf is the plaquette read from one of its corners, so
+//   x:        U_mu(x) (D U_nu(x)^+)            x+mu:  D E
+//   x+mu+nu:  U_mu(x+nu)^+ (E U_nu(x+mu))      x+nu:  E D
+// with D = U_nu(x+mu) U_mu(x+nu)^+ and E = U_nu(x)^+ U_mu(x): 8 products where
+// every site on its own takes 12 for its four leaves.  FP64 arithmetic is the
+// bound, so the anti-Hermitian parts (9 reals) go through memory to the sites
+// they belong to: slots [plane][leaf][9] in the 72 reals of Ahat's record.  With
+// the packed inverse below, qcd_build_clover on 16^3 x 32 went from 3.0 ms (one
+// kernel, its FP64 pipe 91 % busy, matrices in local memory) to 1.1 ms.
+__global__ void __launch_bounds__(128) clover_leaf_kernel(Geom g, const double2* __restrict__ U64, double* slots,
+                                                          int q0) {
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  int mu, nu, x[4];
+  plane_dirs(q0 + blockIdx.y, mu, nu);
+  global_coords(g, (int)(s / g.Vb), (int)(s % g.Vb), x);
+  const long long s1 = site_at(g, x, mu, 1, -1, 0), s2 = site_at(g, x, mu, 1, nu, 1), s3 = site_at(g, x, nu, 1, -1, 0);
+  const int j0 = 36 * blockIdx.y;
+  double t[9];
+  const M3 D = m3mul(link_of(g, U64, s1, nu), m3dag(link_of(g, U64, s3, mu)));
+  {
+    const M3 E = m3mul(m3dag(link_of(g, U64, s, nu)), link_of(g, U64, s, mu));
+    antiherm_product(D, E, t);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) q.m[i][j] = q.m[i][j] + l.m[i][j];
-  // leaf 3: U_mu(x-mu)^+ U_nu(x-mu-nu)^+ U_mu(x-mu-nu) U_nu(x-nu)
-  l = m3mul(m3mul(m3dag(link_at(g, U64, x, mu, -1, 0, mu, nu)), m3dag(link_at(g, U64, x, nu, -1, -1, mu, nu))),
-            m3mul(link_at(g, U64, x, mu, -1, -1, mu, nu), link_at(g, U64, x, nu, 0, -1, mu, nu)));
+    for (int k = 0; k < 9; ++k) *rec_real(slots, g, s1, j0 + 9 + k) = t[k];
+    antiherm_product(E, D, t);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+    for (int k = 0; k < 9; ++k) *rec_real(slots, g, s3, j0 + 27 + k) = t[k];
+    antiherm_product(m3dag(link_of(g, U64, s3, mu)), m3mul(E, link_of(g, U64, s1, nu)), t);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) q.m[i][j] = q.m[i][j] + l.m[i][j];
-  // leaf 4: U_nu(x-nu)^+ U_mu(x-nu) U_nu(x-nu+mu) U_mu(x)^+
-  l = m3mul(m3mul(m3dag(link_at(g, U64, x, nu, 0, -1, mu, nu)), link_at(g, U64, x, mu, 0, -1, mu, nu)),
-            m3mul(link_at(g, U64, x, nu, 1, -1, mu, nu), m3dag(link_at(g, U64, x, mu, 0, 0, mu, nu))));
-  M3 f;
+    for (int k = 0; k < 9; ++k) *rec_real(slots, g, s2, j0 + 18 + k) = t[k];
+  }
+  antiherm_product(link_of(g, U64, s, mu), m3mul(D, m3dag(link_of(g, U64, s, nu))), t);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int k = 0; k < 9; ++k) *rec_real(slots, g, s, j0 + k) = t[k];
+}
+
+// Fhat (9 reals, the form above) of two planes at a site: an eighth of its leaves' sum
+__device__ __forceinline__ void leaf_sum(const double* slots, const Geom& g, long long s, double f[18]) {
+  double2 v[36];
+  const double2* p = (const double2*)rec_real(const_cast<double*>(slots), g, s, 0);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      cd qij = q.m[i][j] + l.m[i][j];
-      f.m[i][j] = qij;
+  for (int k = 0; k < 36; ++k) v[k] = p[(long long)k * g.Vb];
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      double sum = 0;
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {
+        const int j = 36 * q + 9 * l + k;
+        const double w = (j & 1) ? v[j >> 1].y : v[j >> 1].x;
+        sum = l == 0 ? w : sum + w;
+      }
+      f[9 * q + k] = 0.125 * sum;
     }
-  M3 o;
+}
+
+// Fhat of the launch's two planes into reals 18 (q0 / 2) .. + 17 of A's record memory
+__global__ void __launch_bounds__(128) clover_sum_kernel(Geom g, const double* __restrict__ slots, double* F, int q0) {
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  double f[18];
+  leaf_sum(slots, g, s, f);
+  double2* o = (double2*)rec_real(F, g, s, 9 * q0);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) o.m[i][j] = 0.125 * (f.m[i][j] - conjg(f.m[j][i]));
-  return o;
+  for (int k = 0; k < 9; ++k) o[(long long)k * g.Vb] = make_double2(f[2 * k], f[2 * k + 1]);
 }
 
 // pack the Hermitian 6x6 M into 36 reals: 6 diagonal, then (i < j) pairs row-major
@@ -144,68 +210,196 @@ __device__ bool invert6(cd M[6][6], cd Inv[6][6]) {
   return true;
 }
 
-__global__ void clover_build_kernel(Geom g, const double2* __restrict__ U64, double m0, double csw, FieldPtr A,
-                                    FieldPtr Ahat, int* bad) {
-  long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// i times element (a, b) of an anti-Hermitian matrix in 9 reals (Hermitian result)
+__device__ __forceinline__ cd times_i_at(const double f[9], int a, int b) {
+  if (a == b) return {-f[a], 0.0};
+  const int k = 3 + 2 * (a + b - 1);
+  return a < b ? cd{-f[k + 1], f[k]} : cd{-f[k + 1], -f[k]};
+}
+
+// Inverse of a Hermitian 6x6 in packed form by six sweeps: for each pivot k,
+//   B_ij = A_ij - A_ik A_kj / A_kk,  B_ik = A_ik / A_kk,  B_kk = -1 / A_kk,
+// which keeps the matrix Hermitian (60 FP64 operations per pivot where the
+// elimination of M beside a unit matrix takes 288) and leaves minus the
+// inverse.  Takes the pivots on the diagonal in order, as the elimination with
+// column pivoting does whenever each is the largest of its column; returns
+// false otherwise (m is then spoilt and the caller eliminates with pivoting).
+__device__ __forceinline__ int herm_at(int i, int j) {  // packed index of (i < j)'s real part
+  return 6 + 2 * (i * (11 - i) / 2 + (j - i - 1));
+}
+__device__ __forceinline__ bool invert6_sweep(double m[36]) {
+  double scale = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) scale = fmax(scale, fabs(m[i]));
+#pragma unroll
+  for (int k = 6; k < 36; k += 2) scale = fmax(scale, fabs(m[k]) + fabs(m[k + 1]));
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const double piv = fabs(m[k]);
+    ok &= piv > 1e-14 * scale;
+#pragma unroll
+    for (int i = k + 1; i < 6; ++i) ok &= !(fabs(m[herm_at(k, i)]) + fabs(m[herm_at(k, i) + 1]) > piv);
+    const double d = 1.0 / m[k];
+    cd col[6], sc[6];  // A_ik and A_ik / A_kk
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      if (i == k) continue;
+      const int p = i < k ? herm_at(i, k) : herm_at(k, i);
+      col[i] = {m[p], i < k ? m[p + 1] : -m[p + 1]};
+      sc[i] = d * col[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      if (i == k) continue;
+      m[i] = fma(-sc[i].re, col[i].re, fma(-sc[i].im, col[i].im, m[i]));
+#pragma unroll
+      for (int j = i + 1; j < 6; ++j) {  // A_ij -= (A_ik / A_kk) conj(A_jk)
+        if (j == k) continue;
+        const int p = herm_at(i, j);
+        m[p] = fma(-sc[i].re, col[j].re, fma(-sc[i].im, col[j].im, m[p]));
+        m[p + 1] = fma(-sc[i].im, col[j].re, fma(sc[i].re, col[j].im, m[p + 1]));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      if (i == k) continue;
+      const int p = i < k ? herm_at(i, k) : herm_at(k, i);
+      m[p] = sc[i].re;
+      m[p + 1] = i < k ? sc[i].im : -sc[i].im;
+    }
+    m[k] = -d;
+  }
+#pragma unroll
+  for (int k = 0; k < 36; ++k) m[k] = -m[k];
+  return ok;
+}
+
+// the general inverse of a packed Hermitian block (pivoting, matrices in local memory)
+__device__ __noinline__ bool invert6_packed(double* m) {
+  cd M[6][6], Inv[6][6];
+  int k = 6;
+  for (int i = 0; i < 6; ++i) {
+    M[i][i] = {m[i], 0.0};
+    for (int j = i + 1; j < 6; ++j) {
+      M[i][j] = {m[k], m[k + 1]};
+      M[j][i] = conjg(M[i][j]);
+      k += 2;
+    }
+  }
+  const bool ok = invert6(M, Inv);
+  // symmetrise the inverse (Hermitian up to rounding)
+  for (int i = 0; i < 6; ++i)
+    for (int j = i; j < 6; ++j) {
+      const cd a = Inv[i][j], b = conjg(Inv[j][i]);
+      Inv[i][j] = 0.5 * (a + b);
+      Inv[j][i] = conjg(Inv[i][j]);
+    }
+  pack_herm(Inv, m);
+  return ok;
+}
+
+// A and Ahat of a site from Fhat: planes 01, 23, 02, 13 from A's record memory,
+// 03 and 12 from the last leaves in Ahat's; both are then overwritten by the
+// records (a thread reads and writes its own site's reals only)
+__global__ void __launch_bounds__(128) clover_build_kernel(Geom g, double m0, double csw, FieldPtr A, FieldPtr Ahat,
+                                                           int* bad) {
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
-  int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
-  int x[4];
-  global_coords(g, blk, r, x);
-  M3 F01 = fhat(g, U64, x, 0, 1), F02 = fhat(g, U64, x, 0, 2), F03 = fhat(g, U64, x, 0, 3);
-  M3 F12 = fhat(g, U64, x, 1, 2), F13 = fhat(g, U64, x, 1, 3), F23 = fhat(g, U64, x, 2, 3);
+  const int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
+  double f[54];  // [01, 23, 02, 13, 03, 12][9]
+  {
+    const double2* p = (const double2*)rec_real((double*)A.data, g, s, 0);
+#pragma unroll
+    for (int k = 0; k < 18; ++k) {
+      const double2 v = p[(long long)k * g.Vb];
+      f[2 * k] = v.x;
+      f[2 * k + 1] = v.y;
+    }
+    leaf_sum((const double*)Ahat.data, g, s, f + 36);
+  }
   // sigma_0k = diag(s_k, -s_k); sigma_jk = -eps_jkl diag(s_l, s_l).  Hence
   // upper block: (i c/2) sum_k s_k (x) E_k, E = (F01 - F23, F02 + F13, F03 - F12);
   // lower block: -(i c/2) sum_k s_k (x) B_k, B = (F01 + F23, F02 - F13, F03 + F12).
-  double rec[72], inv[72];
+  double2* out = (double2*)A.data + (long long)blk * 36 * g.Vb + r;
+  double2* hat = (double2*)Ahat.data + (long long)blk * 36 * g.Vb + r;
   const bool odd = r >= g.Vbh;
+#pragma unroll 1
   for (int chir = 0; chir < 2; ++chir) {
-    const double sg = chir == 0 ? 1.0 : -1.0;
-    cd M[6][6];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        cd E1 = F01.m[a][b] - sg * F23.m[a][b];
-        cd E2 = F02.m[a][b] + sg * F13.m[a][b];
-        cd E3 = F03.m[a][b] - sg * F12.m[a][b];
-        // s1 E1 + s2 E2 + s3 E3 = [[E3, E1 - i E2], [E1 + i E2, -E3]]
-        cd b00 = E3, b01 = E1 - ti(E2), b10 = E1 + ti(E2), b11 = -E3;
-        const double f = 0.5 * csw * sg;
-        M[a][b] = f * ti(b00);
-        M[a][3 + b] = f * ti(b01);
-        M[3 + a][b] = f * ti(b10);
-        M[3 + a][3 + b] = f * ti(b11);
-      }
-    for (int i = 0; i < 6; ++i) M[i][i].re += 4.0 + m0;
-    pack_herm(M, rec + 36 * chir);
-    if (odd) {
-      cd Inv[6][6];
-      if (!invert6(M, Inv)) atomicExch(bad, 1);
-      // symmetrise the inverse (Hermitian up to rounding)
-      for (int i = 0; i < 6; ++i)
-        for (int j = i; j < 6; ++j) {
-          cd a = Inv[i][j], b = conjg(Inv[j][i]);
-          Inv[i][j] = 0.5 * (a + b);
-          Inv[j][i] = conjg(Inv[i][j]);
-        }
-      pack_herm(Inv, inv + 36 * chir);
+    const double sg = chir == 0 ? 1.0 : -1.0, c = 0.5 * csw * sg;
+    double e[3][9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      e[0][k] = f[k] - sg * f[9 + k];
+      e[1][k] = f[18 + k] + sg * f[27 + k];
+      e[2][k] = f[36 + k] - sg * f[45 + k];
     }
+    // s1 E1 + s2 E2 + s3 E3 = [[E3, E1 - i E2], [E1 + i E2, -E3]], times i c
+    double m[36];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) m[i] = 4.0 + m0 + (i < 3 ? c : -c) * times_i_at(e[2], i % 3, i % 3).re;
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+      for (int j = i + 1; j < 6; ++j) {
+        cd v;
+        if ((i < 3) == (j < 3)) {
+          const cd h = times_i_at(e[2], i % 3, j % 3);
+          v = i < 3 ? h : -h;
+        } else {
+          v = times_i_at(e[0], i, j - 3) + mti(times_i_at(e[1], i, j - 3));
+        }
+        m[herm_at(i, j)] = c * v.re;
+        m[herm_at(i, j) + 1] = c * v.im;
+      }
+#pragma unroll
+    for (int k = 0; k < 18; ++k) out[(long long)(18 * chir + k) * g.Vb] = make_double2(m[2 * k], m[2 * k + 1]);
+    if (odd) {
+      double w[36];
+#pragma unroll
+      for (int k = 0; k < 36; ++k) w[k] = m[k];
+      if (!invert6_sweep(w)) {
+        double t[36];
+#pragma unroll
+        for (int k = 0; k < 36; ++k) t[k] = m[k];
+        if (!invert6_packed(t)) atomicExch(bad, 1);
+#pragma unroll
+        for (int k = 0; k < 36; ++k) w[k] = t[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 36; ++k) m[k] = w[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 18; ++k) hat[(long long)(18 * chir + k) * g.Vb] = make_double2(m[2 * k], m[2 * k + 1]);
   }
-  store_record<P64, 72, double>(A, g.Vb, blk, r, rec);
-  store_record<P64, 72, double>(Ahat, g.Vb, blk, r, odd ? inv : rec);
 }
 
 int build_clover(qcd_ctx* c, cudaStream_t s) {
   if (!c->gauge_loaded) return QCD_ERR_STATE;
   ++c->gen;  // every clover record is reallocated
+  c->clover_built = false;  // A's memory is scratch until the last pass
+  // work still queued on other streams may read the records that are kept (the
+  // memory that is freed waits by itself)
+  QCD_CUDA(cudaDeviceSynchronize());
   for (int p = 0; p < 5; ++p) {
+    if (p == P64 && c->A[p].data && c->Ahat[p].data) continue;  // a new gauge field: the same sizes again
     rec_free(c->A[p]);
     rec_free(c->Ahat[p]);
   }
-  QCD_TRY(rec_alloc(c->A[P64], P64, 72, c->V));
-  QCD_TRY(rec_alloc(c->Ahat[P64], P64, 72, c->V));
+  if (!c->A[P64].data) QCD_TRY(rec_alloc(c->A[P64], P64, 72, c->V));
+  if (!c->Ahat[P64].data) QCD_TRY(rec_alloc(c->Ahat[P64], P64, 72, c->V));
   int* d_bad = (int*)c->d_scalars;
   QCD_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
-  clover_build_kernel<<<(unsigned)((c->V + 127) / 128), 128, 0, s>>>(
-      c->g, (const double2*)c->U[P64], c->p.m0, c->p.csw, c->A[P64].ptr(), c->Ahat[P64].ptr(), d_bad);
+  const unsigned grid = (unsigned)((c->V + 127) / 128);
+  double* slots = (double*)c->Ahat[P64].data;
+  for (int q = 0; q < 6; q += 2) {
+    clover_leaf_kernel<<<dim3(grid, 2), 128, 0, s>>>(c->g, (const double2*)c->U[P64], slots, q);
+    QCD_LAUNCHED();
+    if (q == 4) break;  // the last two planes' leaves are summed by the pass that uses them
+    clover_sum_kernel<<<grid, 128, 0, s>>>(c->g, slots, (double*)c->A[P64].data, q);
+    QCD_LAUNCHED();
+  }
+  clover_build_kernel<<<grid, 128, 0, s>>>(c->g, c->p.m0, c->p.csw, c->A[P64].ptr(), c->Ahat[P64].ptr(), d_bad);
   QCD_LAUNCHED();
   int h = 0;
   QCD_CUDA(cudaMemcpyAsync(&h, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
