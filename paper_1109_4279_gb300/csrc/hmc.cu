@@ -129,16 +129,9 @@ __device__ M3 staple_sum(const Lex& g, const double2* U, long long s, int mu) {
   return v;
 }
 
-// F_a = (beta / 6) Im tr(lambda_a M), M = U_mu(x) V_mu(x); tr(lambda_a M) written out
-__global__ void __launch_bounds__(kThreads) gauge_force_kernel(Lex g, const double2* __restrict__ U, double beta,
-                                                               double* __restrict__ F) {
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= 4 * g.V) return;
-  const long long s = l / 4;
-  const int mu = (int)(l % 4);
-  const M3 M = mmul(mload(U, l), staple_sum(g, U, s, mu));
-  const double f = beta / 6.0, r3 = 0.5773502691896257645;  // 1/sqrt(3)
-  double* o = F + l * 8;
+// o[a] = f Im tr(lambda_a M)
+__device__ __forceinline__ void im_trace_lambda(const M3& M, double f, double o[8]) {
+  const double r3 = 0.5773502691896257645;  // 1/sqrt(3)
   o[0] = f * (M.a[1][0].im + M.a[0][1].im);                         // tr(l1 M) = M10 + M01
   o[1] = f * (M.a[0][1].re - M.a[1][0].re);                         // tr(l2 M) = i (M01 - M10)
   o[2] = f * (M.a[0][0].im - M.a[1][1].im);                         // tr(l3 M) = M00 - M11
@@ -147,6 +140,73 @@ __global__ void __launch_bounds__(kThreads) gauge_force_kernel(Lex g, const doub
   o[5] = f * (M.a[2][1].im + M.a[1][2].im);                         // tr(l6 M) = M21 + M12
   o[6] = f * (M.a[1][2].re - M.a[2][1].re);                         // tr(l7 M) = i (M12 - M21)
   o[7] = f * r3 * (M.a[0][0].im + M.a[1][1].im - 2.0 * M.a[2][2].im);  // tr(l8 M)
+}
+
+// F_a = (beta / 6) Im tr(lambda_a M), M = U_mu(x) V_mu(x): one thread per link
+__global__ void __launch_bounds__(128) gauge_force_kernel(Lex g, const double2* __restrict__ U, double beta,
+                                                          double* __restrict__ F) {
+  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= 4 * g.V) return;
+  double o[8];
+  im_trace_lambda(mmul(mload(U, l), staple_sum(g, U, l / 4, (int)(l % 4))), beta / 6.0, o);
+#pragma unroll
+  for (int a = 0; a < 8; ++a) F[l * 8 + a] = o[a];
+}
+
+// F of link l (+)= sg o
+template <int FIRST>
+__device__ __forceinline__ void force_add(double* F, long long l, double sg, const double o[8]) {
+  double2* f = (double2*)(F + l * 8);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    double2 v = FIRST ? make_double2(0.0, 0.0) : f[k];
+    v.x += sg * o[2 * k];
+    v.y += sg * o[2 * k + 1];
+    f[k] = v;
+  }
+}
+
+// The same force, one thread per plaquette (x; mu < nu).  Read from its corners
+// x, x+mu and x+nu, a plaquette gives every term its four links need:
+//   L1 = U_mu(x) (D U_nu(x)^+)  for U_mu(x) and, negated, U_nu(x),
+//   L2 = D E  for U_nu(x+mu),   L4 = E D, negated, for U_mu(x+nu),
+// D = U_nu(x+mu) U_mu(x+nu)^+, E = U_nu(x)^+ U_mu(x): 6 products per plaquette
+// where the links on their own take 13 x 4 per 6 plaquettes.  Launch (round,
+// colour) takes the plaquettes of two planes without a common direction whose
+// x_mu + x_nu has the colour's parity: those touch every link once, so the sums
+// are plain read-modify-writes in a fixed order; the first launch writes.
+template <int FIRST>
+__global__ void __launch_bounds__(128) gauge_force_plaquette_kernel(Lex g, const double2* __restrict__ U, double f,
+                                                                    int round, int colour, double* __restrict__ F) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (2 * t >= g.V) return;
+  // planes (0 1)(2 3), (0 2)(1 3), (0 3)(1 2)
+  const int mu = blockIdx.y == 0 ? 0 : (round == 0 ? 2 : 1), nu = blockIdx.y == 0 ? round + 1 : (round == 2 ? 2 : 3);
+  int x[4];
+  long long q = t;  // coordinates of the t-th such plaquette: x_nu runs over its half
+#pragma unroll
+  for (int d = 3; d >= 0; --d) {
+    const int n = d == nu ? g.L[d] / 2 : g.L[d];
+    x[d] = (int)(q % n);
+    q /= n;
+  }
+  const int xmu = mu == 0 ? x[0] : (mu == 1 ? x[1] : x[2]);
+#pragma unroll
+  for (int d = 0; d < 4; ++d)
+    if (d == nu) x[d] = 2 * x[d] + ((xmu + colour) & 1);
+  const long long s = g.index(x), s1 = g.shift(s, mu, +1), s3 = g.shift(s, nu, +1);
+  double o[8];
+  const M3 D = mmul(mload(U, s1 * 4 + nu), mdag(mload(U, s3 * 4 + mu)));
+  {
+    const M3 E = mmul(mdag(mload(U, s * 4 + nu)), mload(U, s * 4 + mu));
+    im_trace_lambda(mmul(D, E), f, o);
+    force_add<FIRST>(F, s1 * 4 + nu, 1.0, o);
+    im_trace_lambda(mmul(E, D), f, o);
+    force_add<FIRST>(F, s3 * 4 + mu, -1.0, o);
+  }
+  im_trace_lambda(mmul(mload(U, s * 4 + mu), mmul(D, mdag(mload(U, s * 4 + nu)))), f, o);
+  force_add<FIRST>(F, s * 4 + mu, 1.0, o);
+  force_add<FIRST>(F, s * 4 + nu, -1.0, o);
 }
 
 // per site: sum over mu < nu of (1 - Re tr U_munu / 3); partial sums per CTA
@@ -263,6 +323,13 @@ __global__ void __launch_bounds__(kThreads) sumsq_kernel(long long n, const doub
   cta_sum_store(acc, part);
 }
 
+// Lattices from here on take the gauge force by plaquettes: half the FP64 work, but
+// six launches one after another of about 26 us (a warp's FP64 operation holds its
+// SM quarter's unit for 64 cycles, so that is what the 700 of one thread take).
+// By plaquettes / by links: 4096 sites 158 / 76 us, 8192 161 / 126, 16384 172 / 268,
+// 131072 950 / 1755, 663552 4530 / 8830.
+static constexpr long long kPlaquetteSites = 12288;
+
 static Lex lex_of(qcd_ctx* c) {
   Lex g;
   for (int mu = 0; mu < 4; ++mu) g.L[mu] = c->p.dims[mu];
@@ -330,8 +397,21 @@ extern "C" int qcd_gauge_action(qcd_ctx* c, const double* U, double beta, double
 extern "C" int qcd_gauge_force(qcd_ctx* c, const double* U, double beta, double* F, void* stream) {
   if (!c || !U || !F) return QCD_ERR_ARG;
   const Lex g = lex_of(c);
-  gauge_force_kernel<<<grid_for(4 * g.V), kThreads, 0, (cudaStream_t)stream>>>(g, (const double2*)U, beta, F);
-  QCD_LAUNCHED();
+  const cudaStream_t s = (cudaStream_t)stream;
+  if (g.V < kPlaquetteSites) {
+    // 128 threads: one warp for each quarter of an SM (with 256, 135 us at 4096 sites)
+    gauge_force_kernel<<<(unsigned)((4 * g.V + 127) / 128), 128, 0, s>>>(g, (const double2*)U, beta, F);
+    QCD_LAUNCHED();
+    return QCD_OK;
+  }
+  const dim3 grid((unsigned)((g.V / 2 + 127) / 128), 2);
+  for (int k = 0; k < 6; ++k) {
+    if (k == 0)
+      gauge_force_plaquette_kernel<1><<<grid, 128, 0, s>>>(g, (const double2*)U, beta / 6.0, 0, 0, F);
+    else
+      gauge_force_plaquette_kernel<0><<<grid, 128, 0, s>>>(g, (const double2*)U, beta / 6.0, k / 2, k % 2, F);
+    QCD_LAUNCHED();
+  }
   return QCD_OK;
 }
 
