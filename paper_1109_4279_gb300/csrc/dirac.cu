@@ -358,62 +358,66 @@ __global__ void __launch_bounds__(2 * kPairSites, QCD_PAIR_MIN_CTAS) dirac_pair_
 // times faster on GB300; the result agrees with the FP64 operator to about
 // 2^-46 relative.
 // ------------------------------------------------------------------------
-struct cdf {
-  df re, im;
+//
+// The arithmetic is written on packed FP32x2 instructions, two independent
+// values per instruction: the FP32 lanes are the same, but half the issue slots
+// go by, and issue was what the scalar form ran out of (59 % of the slots, the
+// FMA pipe at 46 %).  In a hop the two lanes are the two rows of the projected
+// spinor (upper spins 0, 1, then lower spins 2, 3), so a link entry serves both;
+// in the clover term they are the real and imaginary part of one component.
+// The order of the operations on every value is that of the scalar form, and
+// so are the results to the last rounding.  32^3 x 64 with an FP32 input: 1.41 ->
+// 1.09 ms, and 0.96 ms with the hops' data asked for ahead in registers (below);
+// on 8^3 x 16 34 -> 17 us.  The FMA pipe alone needs 0.69 ms.
+struct df2 {  // two double-floats
+  float2 hi, lo;
 };
-__device__ __forceinline__ cdf cdf_of(const float4& v) { return {{v.x, v.y}, {v.z, v.w}}; }
-// x + y without the final renormalisation (a valid double-float operand)
-__device__ __forceinline__ df dsum(df x, df y) {
-  df t = two_sum(x.hi, y.hi);
-  t.lo += x.lo + y.lo;
-  return t;
+struct acc2 {  // two running sums (dfacc)
+  float2 s, c;
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// s + e = a + b exactly
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = add2(a, b);
+  const float2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
-__device__ __forceinline__ cdf cplus(const cdf& x, const cdf& y) { return {dsum(x.re, y.re), dsum(x.im, y.im)}; }
-__device__ __forceinline__ cdf cminus(const cdf& x, const cdf& y) {
-  return {dsum(x.re, df_neg(y.re)), dsum(x.im, df_neg(y.im))};
+// a = x y, a += x y for double-floats x, y (x.lo y.lo dropped; YLO: y.lo is not 0)
+template <bool YLO>
+__device__ __forceinline__ void acc2_set(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
+  const float2 p = __fmul2_rn(xh, yh);
+  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
+  if (YLO) e = __ffma2_rn(xh, yl, e);
+  a = {p, e};
 }
-__device__ __forceinline__ cdf ctimes_i(const cdf& z) { return {df_neg(z.im), z.re}; }   // i z
-__device__ __forceinline__ cdf ctimes_mi(const cdf& z) { return {z.im, df_neg(z.re)}; }  // -i z
+template <bool YLO>
+__device__ __forceinline__ void acc2_prod(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
+  const float2 p = __fmul2_rn(xh, yh);
+  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
+  if (YLO) e = __ffma2_rn(xh, yl, e);
+  float2 t;
+  two_sum2(a.s, p, a.s, t);
+  a.c = add2(a.c, add2(t, e));
+}
+// a += f z for f = +-1/2 (exact)
+__device__ __forceinline__ void acc2_add(acc2& a, float2 f, const acc2& z) {
+  float2 t;
+  two_sum2(a.s, __fmul2_rn(f, z.s), a.s, t);
+  a.c = add2(a.c, add2(t, __fmul2_rn(f, z.c)));
+}
 
-// (ar, ai) += u h and (ar, ai) += conj(u) h
-__device__ __forceinline__ void cmac_df(dfacc& ar, dfacc& ai, const cdf& u, const cdf& h) {
-  acc_prod(ar, u.re.hi, u.re.lo, h.re.hi, h.re.lo);
-  acc_prod(ar, -u.im.hi, -u.im.lo, h.im.hi, h.im.lo);
-  acc_prod(ai, u.re.hi, u.re.lo, h.im.hi, h.im.lo);
-  acc_prod(ai, u.im.hi, u.im.lo, h.re.hi, h.re.lo);
-}
-__device__ __forceinline__ void cjmac_df(dfacc& ar, dfacc& ai, const cdf& u, const cdf& h) {
-  acc_prod(ar, u.re.hi, u.re.lo, h.re.hi, h.re.lo);
-  acc_prod(ar, u.im.hi, u.im.lo, h.im.hi, h.im.lo);
-  acc_prod(ai, u.re.hi, u.re.lo, h.im.hi, h.im.lo);
-  acc_prod(ai, -u.im.hi, -u.im.lo, h.re.hi, h.re.lo);
-}
-
+// the 24 output reals of a site: [spin pair][colour], lanes = the pair's spins
 struct SpinAcc {
-  dfacc re[4][3], im[4][3];
+  acc2 re[2][3], im[2][3];
 };
-
-// acc[s][c] += f z for f = +-1/2 (exact) and a lazily summed z = (zr, zi)
-__device__ __forceinline__ void acc_cadd(SpinAcc& a, int s, int c, float f, const dfacc& zr, const dfacc& zi) {
-  acc_add(a.re[s][c], f * zr.s, f * zr.c);
-  acc_add(a.im[s][c], f * zi.s, f * zi.c);
-}
-// acc[s][c] += f i z
-__device__ __forceinline__ void acc_cadd_i(SpinAcc& a, int s, int c, float f, const dfacc& zr, const dfacc& zi) {
-  acc_add(a.re[s][c], -f * zi.s, -f * zi.c);
-  acc_add(a.im[s][c], f * zr.s, f * zr.c);
+// real (part 0) or imaginary part of component (spin, colour) as a double-float
+__device__ __forceinline__ df acc_real(const SpinAcc& a, int sp, int c, int part) {
+  const acc2& v = part ? a.im[sp >> 1][c] : a.re[sp >> 1][c];
+  return (sp & 1) ? two_sum(v.s.y, v.c.y) : two_sum(v.s.x, v.c.x);
 }
 
-// z times a phase +-1 or +-i: (im ? i z : z) * sg
-__device__ __forceinline__ cdf cphase(const cdf& z, bool im, float sg) {
-  const df re = im ? df_neg(z.im) : z.re, imv = im ? z.re : z.im;
-  return {{sg * re.hi, sg * re.lo}, {sg * imv.hi, sg * imv.lo}};
-}
-
-// The eight hops share one loop body (direction, projection sign and link
-// conjugation chosen at run time), and the two clover blocks another: the
-// double-float arithmetic is long, and unrolled over every hop it would not
-// fit the instruction cache.
 // what a double-float hop needs to find its neighbour: the site's in-block
 // lexicographic index, its packed local coordinates (8 bits each), its block
 // coordinates (16 bits each) and its parity; kept in five registers (a table
@@ -472,39 +476,141 @@ __device__ __forceinline__ void df_hop_nbr(const Geom& g, int blk, const DfSite&
   cf = wrap ? -0.5f * g.bcf[mu] : -0.5f;
 }
 
-// complex q (= 3 spin + colour) of site (blk, r) of a spinor field as a
-// double-float pair: from a double-float field (chunk q holds re hi, re lo, im
-// hi, im lo) or, IN32, from an FP32 field (chunk q / 2 holds complexes 2 (q / 2)
-// and 2 (q / 2) + 1; the low parts are 0)
+__device__ __forceinline__ float2 lane_swap(float2 v) { return make_float2(v.y, v.x); }
+__device__ __forceinline__ void lane_swap(acc2& a) {
+  a.s = lane_swap(a.s);
+  a.c = lane_swap(a.c);
+}
+
+// What a hop reads, in registers: the neighbour's spinor record (double-float:
+// (re hi, re lo, im hi, im lo) per complex number 3 spin + colour; IN32: two
+// complex numbers per chunk, the low parts being 0) and the link's rows (of the
+// transposed link for a backward hop).  A hop's data are asked for while the
+// hop before it computes, each piece as soon as its registers are free: waiting
+// for them was the largest stall (4.9 of 9.2 cycles per issue), also with the
+// next hop's lines prefetched to L1.
 template <bool IN32>
-__device__ __forceinline__ cdf df_load(const float4* __restrict__ f, int Vb, int blk, int r, int q) {
-  if constexpr (IN32) {
-    const float2 v = __ldg((const float2*)(f + ((long long)blk * 6 + (q >> 1)) * Vb + r) + (q & 1));
-    return cdf{df{v.x, 0.f}, df{v.y, 0.f}};
-  } else {
-    return cdf_of(__ldg(f + ((long long)blk * 12 + q) * Vb + r));
+struct DfHopData {
+  static constexpr int NQ = IN32 ? 6 : 12;
+  float4 p[NQ], u[9];
+  const float4 *fp, *up;
+  int sa, sb;
+  float cf;  // -1/2, times the boundary sign where the hop wraps around
+  __device__ __forceinline__ void locate(const Geom& g, const float4* __restrict__ U, const float4* __restrict__ fin,
+                                         int blk, int r, const DfSite& ds, int h) {
+    int hb, hr;
+    df_hop_nbr(g, blk, ds, h, hb, hr, cf);
+    const int mu = h >> 1, bwd = h & 1;
+    fp = fin + (long long)hb * NQ * g.Vb + hr;
+    up = U + ((long long)((bwd ? hb : blk) * 4 + mu) * 9) * g.Vb + (bwd ? hr : r);
+    sa = bwd ? g.Vb : 3 * g.Vb;
+    sb = bwd ? 3 * g.Vb : g.Vb;
+  }
+  __device__ __forceinline__ void load_spinor(int Vb) {
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) p[k] = __ldg(fp + (long long)k * Vb);
+  }
+  __device__ __forceinline__ void load_row(int a) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) u[3 * a + b] = __ldg(up + a * sa + b * sb);
+  }
+  // real (part 0) or imaginary part of the components (spin s0, colour a), (spin s1, colour a)
+  __device__ __forceinline__ df2 pair(int s0, int s1, int a, int part) const {
+    const int c0 = 3 * s0 + a, c1 = 3 * s1 + a;
+    if constexpr (IN32) {
+      const float4 x = p[c0 >> 1], y = p[c1 >> 1];
+      const float vx = (c0 & 1) ? (part ? x.w : x.z) : (part ? x.y : x.x);
+      const float vy = (c1 & 1) ? (part ? y.w : y.z) : (part ? y.y : y.x);
+      return {make_float2(vx, vy), bc2(0.f)};
+    } else {
+      const float4 x = p[c0], y = p[c1];
+      return part ? df2{make_float2(x.z, y.z), make_float2(x.w, y.w)}
+                  : df2{make_float2(x.x, y.x), make_float2(x.y, y.y)};
+    }
+  }
+};
+
+// one hop in direction MU: forward (bwd = 0) or backward, S = -1 for the
+// projector 1 - g, +1 for 1 + g; d holds its data and is refilled for the next
+// hop (located by `next`) on the way.  In directions 1 and 2 the upper rows 0, 1
+// pair with spins 3, 2: there the lower lanes of acc are (3, 2), swapped by the
+// caller.  U^+ h = conj(U^T conj(h)): a backward hop conjugates h and the result.
+template <int MU, bool IN32, typename Next>
+__device__ __forceinline__ void df_hop(DfHopData<IN32>& d, int Vb, int bwd, float S, bool more, Next next,
+                                       SpinAcc& acc) {
+  constexpr bool kSwap = MU == 1 || MU == 2, kImag = MU == 1 || MU == 3;
+  const float cj = bwd ? -1.f : 1.f, cf = d.cf;
+  df2 hre[3], him[3];
+  {
+    // q = S (phase) p_lower: phases (-1, -1), (-i, -i), (-1, +1), (-i, +i) for MU = 0 .. 3
+    const float s1 = MU >= 2 ? -S : S;  // lane 1 has the opposite sign in directions 2, 3
+    const float2 qr = kImag ? make_float2(S, s1) : make_float2(-S, -s1), qi = make_float2(-S, -s1);
+    constexpr int l0 = kSwap ? 3 : 2, l1 = kSwap ? 2 : 3;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const df2 ur = d.pair(0, 1, a, 0), ui = d.pair(0, 1, a, 1);
+      const df2 lr = d.pair(l0, l1, a, kImag ? 1 : 0), li = d.pair(l0, l1, a, kImag ? 0 : 1);
+      two_sum2(ur.hi, __fmul2_rn(qr, lr.hi), hre[a].hi, hre[a].lo);
+      two_sum2(ui.hi, __fmul2_rn(qi, li.hi), him[a].hi, him[a].lo);
+      if (!IN32) {
+        hre[a].lo = add2(hre[a].lo, add2(ur.lo, __fmul2_rn(qr, lr.lo)));
+        him[a].lo = add2(him[a].lo, add2(ui.lo, __fmul2_rn(qi, li.lo)));
+      }
+      him[a].hi = __fmul2_rn(bc2(cj), him[a].hi);
+      him[a].lo = __fmul2_rn(bc2(cj), him[a].lo);
+    }
+  }
+  if (more) {
+    next();
+    d.load_spinor(Vb);
+  }
+  const float2 fu = bc2(cf), fui = bc2(cj * cf);
+  // the lower rows get conj(phase) S w: factors of their real and imaginary part
+  const float fl0 = MU == 0 || MU == 2 ? -S * cf : S * cf, fl1 = MU >= 2 ? -fl0 : fl0;
+  const float2 fl = make_float2(fl0, fl1), flj = make_float2(cj * fl0, cj * fl1);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    acc2 wr, wi;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const float4 u = d.u[3 * a + b];
+      if (b == 0)
+        acc2_set<true>(wr, bc2(u.x), bc2(u.y), hre[b].hi, hre[b].lo);
+      else
+        acc2_prod<true>(wr, bc2(u.x), bc2(u.y), hre[b].hi, hre[b].lo);
+      acc2_prod<true>(wr, bc2(-u.z), bc2(-u.w), him[b].hi, him[b].lo);
+      if (b == 0)
+        acc2_set<true>(wi, bc2(u.x), bc2(u.y), him[b].hi, him[b].lo);
+      else
+        acc2_prod<true>(wi, bc2(u.x), bc2(u.y), him[b].hi, him[b].lo);
+      acc2_prod<true>(wi, bc2(u.z), bc2(u.w), hre[b].hi, hre[b].lo);
+    }
+    if (more) d.load_row(a);
+    acc2_add(acc.re[0][a], fu, wr);
+    acc2_add(acc.im[0][a], fui, wi);
+    if (kImag) {  // times i
+      acc2_add(acc.re[1][a], neg2(flj), wi);
+      acc2_add(acc.im[1][a], fl, wr);
+    } else {
+      acc2_add(acc.re[1][a], fl, wr);
+      acc2_add(acc.im[1][a], flj, wi);
+    }
   }
 }
 
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
-
-// the lines hop h reads (the neighbour's spinor and the link) asked for in L1
-// one hop ahead: the arithmetic of a hop is long, and the gathers of the next
-// one then find their lines near instead of waiting a DRAM round trip
-template <bool IN32>
-__device__ __forceinline__ void df_prefetch_hop(const Geom& g, const float4* __restrict__ U,
-                                                const float4* __restrict__ fin, int blk, int r, const DfSite& ds,
-                                                int h) {
-  int hb, hr;
-  float cf;
-  df_hop_nbr(g, blk, ds, h, hb, hr, cf);
-  constexpr int NQ = IN32 ? 6 : 12;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) prefetch_l1(fin + ((long long)hb * NQ + q) * g.Vb + hr);
-  const int mu = h >> 1, bwd = h & 1;
-  const float4* ud = U + ((long long)((bwd ? hb : blk) * 4 + mu) * 9) * g.Vb + (bwd ? hr : r);
-#pragma unroll
-  for (int k = 0; k < 9; ++k) prefetch_l1(ud + (long long)k * g.Vb);
+template <int MU, int DAG, bool IN32>
+__device__ __forceinline__ void df_hop_pair(const Geom& g, const float4* __restrict__ U,
+                                            const float4* __restrict__ fin, int blk, int r, const DfSite& ds,
+                                            DfHopData<IN32>& d, SpinAcc& acc) {
+  constexpr float SF = DAG ? 1.f : -1.f;  // D: (1 - g) psi(x + mu); D^+: (1 + g) psi(x + mu)
+  // the two hops of a direction share their code (its four copies fit the
+  // instruction cache; eight of the scalar form did not: no_instruction stalls
+  // of 8.6 per issue)
+#pragma unroll 1
+  for (int bwd = 0; bwd < 2; ++bwd) {
+    const int h = 2 * MU + bwd;
+    df_hop<MU, IN32>(d, g.Vb, bwd, bwd ? -SF : SF, h < 7, [&] { d.locate(g, U, fin, blk, r, ds, h + 1); }, acc);
+  }
 }
 
 // (D psi)(x) (D^+ with DAG) at site (blk, r) of the field fin (double-float,
@@ -513,110 +619,87 @@ template <int DAG, bool IN32 = false>
 __device__ __forceinline__ void df_site(const Geom& g, const float4* __restrict__ U, const FieldPtr& A,
                                         const float4* __restrict__ fin, int blk, int r, const DfSite& ds,
                                         SpinAcc& acc) {
-  constexpr float SF = DAG ? 1.f : -1.f;  // D: (1 - g) psi(x + mu); D^+: (1 + g) psi(x + mu)
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp)
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) acc.re[sp][c] = acc.im[sp][c] = dfacc{0.f, 0.f};
-#pragma unroll 1
-  for (int h = 0; h < 8; ++h) {
-    const int mu = h >> 1, bwd = h & 1;
-    int hb, hr;
-    float cf;
-    df_hop_nbr(g, blk, ds, h, hb, hr, cf);
-    if (h < 7) df_prefetch_hop<IN32>(g, U, fin, blk, r, ds, h + 1);
-    // chiral-basis projection (1 + S g_mu): h_i = p_i + S ph_i p_{sigma_i}, with
-    // sigma = (2, 3) or (3, 2) and phases -1 / -i (see SpinDir)
-    const bool swap = mu == 1 || mu == 2;
-    const bool im0 = mu == 1 || mu == 3, im1 = im0;
-    const float sg0 = -1.f, sg1 = (mu >= 2) ? 1.f : -1.f;
-    const float S = bwd ? -SF : SF;
-    cdf hh[2][3];
-    {
+    for (int c = 0; c < 3; ++c) acc.re[h][c] = acc.im[h][c] = acc2{bc2(0.f), bc2(0.f)};
+  DfHopData<IN32> d;
+  d.locate(g, U, fin, blk, r, ds, 0);
+  d.load_spinor(g.Vb);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const cdf p0 = df_load<IN32>(fin, g.Vb, hb, hr, a), p1 = df_load<IN32>(fin, g.Vb, hb, hr, 3 + a);
-        const cdf p2 = df_load<IN32>(fin, g.Vb, hb, hr, 6 + a), p3 = df_load<IN32>(fin, g.Vb, hb, hr, 9 + a);
-        hh[0][a] = cplus(p0, cphase(swap ? p3 : p2, im0, S * sg0));
-        hh[1][a] = cplus(p1, cphase(swap ? p2 : p3, im1, S * sg1));
-      }
-    }
-    // w = U h (forward, the site's link) or U^+ h (backward, the neighbour's link)
-    const float4* ud = U + ((long long)((bwd ? hb : blk) * 4 + mu) * 9) * g.Vb + (bwd ? hr : r);
-    const float cj = bwd ? -1.f : 1.f;
-    dfacc wr[2][3], wi[2][3];
+  for (int a = 0; a < 3; ++a) d.load_row(a);
+  df_hop_pair<0, DAG, IN32>(g, U, fin, blk, r, ds, d, acc);
 #pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) wr[sp][a] = wi[sp][a] = dfacc{0.f, 0.f};
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        cdf u = cdf_of(__ldg(ud + (long long)(bwd ? 3 * b + a : 3 * a + b) * g.Vb));
-        u.im = {cj * u.im.hi, cj * u.im.lo};
-#pragma unroll
-        for (int sp = 0; sp < 2; ++sp) cmac_df(wr[sp][a], wi[sp][a], u, hh[sp][b]);
-      }
-    // acc += cf [w ; S B^+ w]: B^+ w has components conj(ph_i) w_i on spins sigma_i
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      acc_cadd(acc, 0, a, cf, wr[0][a], wi[0][a]);
-      acc_cadd(acc, 1, a, cf, wr[1][a], wi[1][a]);
-      // l_i = S cf conj(ph_i) w_i: conj of a real phase is itself, of -i is +i
-      const float f0 = S * cf * (im0 ? -sg0 : sg0), f1 = S * cf * (im1 ? -sg1 : sg1);
-      dfacc l0r = wr[0][a], l0i = wi[0][a], l1r = wr[1][a], l1i = wi[1][a];
-      if (im0) {  // times i: (re, im) -> (-im, re)
-        l0r = {-wi[0][a].s, -wi[0][a].c};
-        l0i = wr[0][a];
-        l1r = {-wi[1][a].s, -wi[1][a].c};
-        l1i = wr[1][a];
-      }
-      acc_cadd(acc, 2, a, swap ? f1 : f0, swap ? l1r : l0r, swap ? l1i : l0i);
-      acc_cadd(acc, 3, a, swap ? f0 : f1, swap ? l0r : l1r, swap ? l0i : l1i);
-    }
+  for (int c = 0; c < 3; ++c) {
+    lane_swap(acc.re[1][c]);
+    lane_swap(acc.im[1][c]);
   }
+  df_hop_pair<1, DAG, IN32>(g, U, fin, blk, r, ds, d, acc);
+  df_hop_pair<2, DAG, IN32>(g, U, fin, blk, r, ds, d, acc);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    lane_swap(acc.re[1][c]);
+    lane_swap(acc.im[1][c]);
+  }
+  df_hop_pair<3, DAG, IN32>(g, U, fin, blk, r, ds, d, acc);
   // clover: two Hermitian 6x6 chiral blocks (6 diagonal reals, then the 15
-  // upper off-diagonal elements), record chunk 18 hb + j = reals 36 hb + 2 j, + 1
+  // upper off-diagonal elements), record chunk 18 hb + j = reals 36 hb + 2 j, + 1;
+  // lanes (re, im)
   const float4* ca = (const float4*)A.data + (long long)blk * 36 * g.Vb + r;
 #pragma unroll 1
   for (int hb = 0; hb < 2; ++hb) {
-    cdf psi[6];
+    df2 psi[6], rot[6];  // psi and i psi
+    if constexpr (IN32) {
+      const float4* p = fin + ((long long)blk * 6 + 3 * hb) * g.Vb + r;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) psi[i] = df_load<IN32>(fin, g.Vb, blk, r, 6 * hb + i);
-    dfacc tr[6], ti[6];
+      for (int k = 0; k < 3; ++k) {
+        const float4 v = __ldg(p + (long long)k * g.Vb);
+        psi[2 * k].hi = make_float2(v.x, v.y);
+        psi[2 * k + 1].hi = make_float2(v.z, v.w);
+      }
+    } else {
+      const float4* p = fin + ((long long)blk * 12 + 6 * hb) * g.Vb + r;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) tr[i] = ti[i] = dfacc{0.f, 0.f};
+      for (int k = 0; k < 6; ++k) {
+        const float4 v = __ldg(p + (long long)k * g.Vb);
+        psi[k] = {make_float2(v.x, v.z), make_float2(v.y, v.w)};
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      rot[k].hi = make_float2(-psi[k].hi.y, psi[k].hi.x);
+      if (!IN32) rot[k].lo = make_float2(-psi[k].lo.y, psi[k].lo.x);
+    }
+    acc2 t[6];
 #pragma unroll
     for (int i = 0; i < 6; i += 2) {  // diagonal reals i, i + 1
       const float4 dv = __ldg(ca + (long long)(18 * hb + i / 2) * g.Vb);
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int ii = i + q;
-        const float dh = q ? dv.z : dv.x, dl = q ? dv.w : dv.y;
-        acc_prod(tr[ii], dh, dl, psi[ii].re.hi, psi[ii].re.lo);
-        acc_prod(ti[ii], dh, dl, psi[ii].im.hi, psi[ii].im.lo);
-      }
+      acc2_set<!IN32>(t[i], bc2(dv.x), bc2(dv.y), psi[i].hi, psi[i].lo);
+      acc2_set<!IN32>(t[i + 1], bc2(dv.z), bc2(dv.w), psi[i + 1].hi, psi[i + 1].lo);
     }
     int kk = 3;
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
       for (int j = i + 1; j < 6; ++j) {
-        const cdf a = cdf_of(__ldg(ca + (long long)(18 * hb + kk) * g.Vb));
+        const float4 a = __ldg(ca + (long long)(18 * hb + kk) * g.Vb);
         ++kk;
-        cmac_df(tr[i], ti[i], a, psi[j]);
-        cjmac_df(tr[j], ti[j], a, psi[i]);
+        acc2_prod<!IN32>(t[i], bc2(a.x), bc2(a.y), psi[j].hi, psi[j].lo);
+        acc2_prod<!IN32>(t[i], bc2(a.z), bc2(a.w), rot[j].hi, rot[j].lo);
+        acc2_prod<!IN32>(t[j], bc2(a.x), bc2(a.y), psi[i].hi, psi[i].lo);
+        acc2_prod<!IN32>(t[j], bc2(-a.z), bc2(-a.w), rot[i].hi, rot[i].lo);
       }
-    // into spins 2 hb, 2 hb + 1
+    // into spins 2 hb (components 0 .. 2) and 2 hb + 1 (3 .. 5)
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
+    for (int c = 0; c < 3; ++c) {
+      const acc2 zr = {make_float2(t[c].s.x, t[c + 3].s.x), make_float2(t[c].c.x, t[c + 3].c.x)};
+      const acc2 zi = {make_float2(t[c].s.y, t[c + 3].s.y), make_float2(t[c].c.y, t[c + 3].c.y)};
       if (hb == 0) {
-        acc_add(acc.re[i / 3][i % 3], tr[i].s, tr[i].c);
-        acc_add(acc.im[i / 3][i % 3], ti[i].s, ti[i].c);
+        acc2_add(acc.re[0][c], bc2(1.f), zr);
+        acc2_add(acc.im[0][c], bc2(1.f), zi);
       } else {
-        acc_add(acc.re[2 + i / 3][i % 3], tr[i].s, tr[i].c);
-        acc_add(acc.im[2 + i / 3][i % 3], ti[i].s, ti[i].c);
+        acc2_add(acc.re[1][c], bc2(1.f), zr);
+        acc2_add(acc.im[1][c], bc2(1.f), zi);
       }
     }
   }
@@ -626,7 +709,7 @@ __device__ __forceinline__ void df_site(const Geom& g, const float4* __restrict_
 // IN32: the input is an FP32 field (an FP32-exact operand, e.g. a preconditioner
 // output), read at half the bytes; the arithmetic is the same
 template <int DAG, bool IN32>
-__global__ void __launch_bounds__(256, 2) dirac_df_kernel(Geom g, const float4* __restrict__ U, FieldPtr A,
+__global__ void __launch_bounds__(256, 1) dirac_df_kernel(Geom g, const float4* __restrict__ U, FieldPtr A,
                                                           FieldPtr in, FieldPtr out, int nrhs,
                                                           const int* __restrict__ mask) {
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -643,7 +726,7 @@ __global__ void __launch_bounds__(256, 2) dirac_df_kernel(Geom g, const float4* 
     float4* o = fout + (long long)blk * 12 * g.Vb + r;
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-      const df re = acc_df(acc.re[q / 3][q % 3]), im = acc_df(acc.im[q / 3][q % 3]);
+      const df re = acc_real(acc, q / 3, q % 3, 0), im = acc_real(acc, q / 3, q % 3, 1);
       o[(long long)q * g.Vb] = make_float4(re.hi, re.lo, im.hi, im.lo);
     }
   }
@@ -667,7 +750,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // arithmetic (as dirac_df_kernel), the difference and |r|^2 in FP64;
 // partial[blockIdx.x] = sum |r|^2 over the CTA, blockIdx.y a right-hand side
 // of a batch (fields V sites apart, partial sums ps doubles apart)
-__global__ void __launch_bounds__(256, 2) residual_df_kernel(Geom g, const float4* __restrict__ U, FieldPtr A,
+__global__ void __launch_bounds__(kDfThreads, 2) residual_df_kernel(Geom g, const float4* __restrict__ U, FieldPtr A,
                                                              FieldPtr b, FieldPtr x, FieldPtr r_out, double* partial,
                                                              long long ps, const int* __restrict__ mask) {
   __shared__ double sh[32];
@@ -687,8 +770,8 @@ __global__ void __launch_bounds__(256, 2) residual_df_kernel(Geom g, const float
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
       const double2 bv = __ldg(bb + e + (long long)q * g.Vb);
-      const double2 v = make_double2(bv.x - df_to_f64(acc_df(acc.re[q / 3][q % 3])),
-                                     bv.y - df_to_f64(acc_df(acc.im[q / 3][q % 3])));
+      const double2 v = make_double2(bv.x - df_to_f64(acc_real(acc, q / 3, q % 3, 0)),
+                                     bv.y - df_to_f64(acc_real(acc, q / 3, q % 3, 1)));
       rr[e + (long long)q * g.Vb] = v;
       nrm = fma(v.x, v.x, fma(v.y, v.y, nrm));
     }
@@ -856,11 +939,11 @@ int residual_df(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec&
   QCD_TRY(ensure_gauge(c, PDF, s));
   QCD_TRY(ensure_clover(c, PDF, s));
   if (!presplit) QCD_TRY(blas_df_split(c, (const double*)x.data, (float*)tmp.data, s, B));
-  const unsigned grid = (unsigned)((c->V + 255) / 256);
+  const unsigned grid = (unsigned)((c->V + kDfThreads - 1) / kDfThreads);
   {
     ProfScope ps(c, QCD_KERNEL_RESIDUAL, s, (bytes_per_site(P64) + 192) * (double)c->V * B.n,
                  1848.0 * (double)c->V * B.n);
-    residual_df_kernel<<<dim3(grid, B.n), 256, 0, s>>>(c->g, (const float4*)c->U[PDF], c->A[PDF].ptr(), b.ptr(),
+    residual_df_kernel<<<dim3(grid, B.n), kDfThreads, 0, s>>>(c->g, (const float4*)c->U[PDF], c->A[PDF].ptr(), b.ptr(),
                                                         tmp.ptr(), r.ptr(), part, B.ps, B.mask);
     QCD_LAUNCHED();
   }

@@ -41,6 +41,10 @@ inline int chunks(int prec, int nreal) {
   return (nreal + w - 1) / w;
 }
 
+// CTA size of the double-float kernels: their registers allow 8 warps per SM, and
+// two CTAs of four fill an SM's gaps better than one of eight
+static constexpr int kDfThreads = 128;
+
 // a device field of N-real records per site in one precision
 struct Rec {
   int prec = -1;
@@ -174,7 +178,7 @@ struct qcd_ctx {
   qcd::Timer timers[QCD_KERNEL_COUNT];
   std::vector<cudaEvent_t> event_pool;
   // launch shape chosen by the autotuner
-  int dirac_threads[5] = {256, 256, 256, 256, 256};  // CTA size of the operator kernel per precision
+  int dirac_threads[5] = {256, 256, 256, 256, qcd::kDfThreads};  // CTA size of the operator kernel per precision
   int sap_rt = 0;  // right-hand sides per CTA of batched SAP launches (0: sap_tile's default)
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)
   double* d_scalars = nullptr;  // small device array for coefficients
