@@ -148,6 +148,8 @@ int qcd_create(qcd_ctx** out, const qcd_params* p) {
   if (!c) return QCD_ERR_NOMEM;
   c->p = *p;
   int st = setup_geometry(c);
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   if (st == QCD_OK) {
     if (cudaMalloc(&c->d_scalars, 64 * 1024) != cudaSuccess || cudaMallocHost(&c->h_scalars, 64 * 1024) != cudaSuccess ||
         cudaMemset(c->d_scalars, 0, 64 * 1024) != cudaSuccess)

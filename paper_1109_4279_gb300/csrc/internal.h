@@ -160,6 +160,7 @@ struct qcd_ctx {
   int* d_tables = nullptr;
   long long V = 0;
   int nblk = 0;
+  int sms = 152;  // SMs of the device the context was created on
   bool gauge_loaded = false, clover_built = false;
   // gauge field and clover in each storage precision (built lazily); index
   // PDF: the double-float copies of the df64 operator

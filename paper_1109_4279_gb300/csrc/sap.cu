@@ -52,6 +52,7 @@ struct SapArgs {
   int* err;             // set to 1 if a staging wait timed out
   long long wait_cycles;  // budget of the staging wait (clock cycles)
   int extra_tx;         // bytes the staging barrier expects beyond the copies (0; a test sets more)
+  int wave;             // CTAs that run at the same time (all SMs)
   // right-hand sides: nrhs fields back to back in eta, rho, psi, out and the
   // face buffers (byte strides below; rho_ns: floats between 16-bit scale
   // arrays); CTA (x, y) solves block x for right-hand sides y rt .. y rt + rt - 1
@@ -307,6 +308,26 @@ __device__ __forceinline__ void prefetch_late_reads(const SapArgs& a, const void
   }
 }
 
+// The CTAs of a wave run in step, so that all SMs would read their next blocks'
+// fields at the same moment (200 KB each: 4 us at the HBM rate) and leave HBM idle
+// while they compute.  During the MR steps a warp asks for the fields of the block
+// that will follow on this SM in L2: 5 % of a launch with one CTA per SM.
+__device__ __forceinline__ void prefetch_next_block(const SapArgs& a) {
+  const Geom& g = a.g;
+  const int next = blockIdx.x + a.wave, lane = threadIdx.x & 31, Vb = g.Vb;
+  if (next >= (int)gridDim.x) return;
+  int blk = 2 * next, n[4];
+  block_coords(g, blk, n);
+  if (((n[0] + n[1] + n[2] + n[3]) & 1) != a.colour) ++blk;
+  const char* links = (const char*)a.U + (size_t)blk * 96 * Vb;
+  const char* clover = (const char*)a.Ahat.data + (size_t)blk * 144 * Vb;
+  for (int o = lane * 4096; o < 96 * Vb; o += 32 * 4096) prefetch_l2(links + o, min(4096, 96 * Vb - o));
+  for (int o = lane * 4096; o < 144 * Vb; o += 32 * 4096) prefetch_l2(clover + o, min(4096, 144 * Vb - o));
+  if (lane == 0) prefetch_l2(a.Ahat.norm + (size_t)blk * Vb, 4 * Vb);
+  if (!a.read_eta && lane < 3)  // the residual's even sites
+    prefetch_l2((const char*)a.rho.data + ((size_t)blk * 3 + lane) * 16 * Vb, 8 * Vb);
+}
+
 // rebuild the compressed 16-bit links of the landing zone (rows 0-1, layout of
 // the storage format) into full 16-bit matrices (HalfExpStage layout)
 template <int P>
@@ -466,6 +487,20 @@ __device__ __forceinline__ Half<T> half_axpy(const Half<T>& a, const Half<T>& b,
   return o;
 }
 
+// (v, w) and |v|^2 of two halves
+template <typename T>
+__device__ __forceinline__ void half_dots(const Half<T>& v, const Half<T>& w, T& re, T& im, T& vv) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const cpx<T> a = v.c[s][c], b = w.c[s][c];
+      re += a.re * b.re + a.im * b.im;
+      im += a.re * b.im - a.im * b.re;
+      vv += a.re * a.re + a.im * a.im;
+    }
+}
+
 // clover chiral block hf applied to an owned half
 template <typename T>
 __device__ __forceinline__ Half<T> clover_half_apply(const T* c36, const Half<T>& in) {
@@ -577,25 +612,6 @@ __device__ __forceinline__ Half<T> pair_reduce_s(const Spinor<T>& acc, int hf, i
   return half_axpy(half_of(acc, hf), s_half(xb, np, i, 1 - hf), T(1));
 }
 
-// full spinor from the owned halves of a pair (ends with a barrier, so the
-// buffer can be reused at once)
-template <typename T>
-__device__ __forceinline__ Spinor<T> pair_full_s(const Half<T>& own, int hf, int i, int np, T* xb) {
-  s_half_store(xb, np, i, hf, own);
-  __syncthreads();
-  const Half<T> o = s_half(xb, np, i, 1 - hf);
-  __syncthreads();
-  Spinor<T> v;
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      v.c[s][c] = hf ? o.c[s][c] : own.c[s][c];
-      v.c[2 + s][c] = hf ? own.c[s][c] : o.c[s][c];
-    }
-  return v;
-}
-
 // owned half of -1/2 (sum of hops) at site r
 template <typename T, typename ST>
 __device__ __forceinline__ Half<T> block_hops(const ST& st, int n, int r, const T* src, const int pk[2], int off,
@@ -608,36 +624,37 @@ __device__ __forceinline__ Half<T> block_hops(const ST& st, int n, int r, const 
   return h;
 }
 
-// deterministic CTA-wide sum of 3 values; every thread gets the totals.  The
-// caller must pass another barrier before the next call.
+// deterministic CTA-wide sum of 3 values in two halves: every warp leaves its sums
+// in red; after a barrier every thread gets the totals
 template <typename T>
-__device__ __forceinline__ void cta_sum3(T& a, T& b, T& c, T* red) {
+__device__ __forceinline__ void sum3_put(T a, T b, T c, T* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
     c += __shfl_xor_sync(0xffffffffu, c, o);
   }
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int w = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0) {
     red[3 * w] = a;
     red[3 * w + 1] = b;
     red[3 * w + 2] = c;
   }
-  __syncthreads();
-  // lane k of every warp takes warp k's partial sums; a butterfly over the
-  // lanes leaves every thread the totals, summed in the same order everywhere
-  const int l = threadIdx.x & 31;
+}
+template <typename T>
+__device__ __forceinline__ void sum3_get(T& a, T& b, T& c, const T* red) {
+  // lane k of every warp takes warp k's sums (at most 16 warps); a butterfly over
+  // 16 lanes leaves every thread the totals, summed in the same order everywhere
+  const int l = threadIdx.x & 15, nw = blockDim.x >> 5;
   a = l < nw ? red[3 * l] : T(0);
   b = l < nw ? red[3 * l + 1] : T(0);
   c = l < nw ? red[3 * l + 2] : T(0);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 8; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
     c += __shfl_xor_sync(0xffffffffu, c, o);
   }
-  // no closing barrier: red is written again only after later barriers
 }
 
 // psi storage precision of the SAP accumulator
@@ -753,68 +770,180 @@ __device__ __forceinline__ Half<float> g_half16(const FieldPtr& f, int Vb, int b
   return h;
 }
 
-// receive the other colour's face contributions at site (blk, r) for the
-// directions of this thread; returns a partial full spinor.  A site lies on at
-// most one face per direction (block extents are at least 2), so one read per
-// direction serves both kinds of face, and a warp waits for one read per
-// direction however its sites split between the kinds.
-template <typename T, typename ST>
-__device__ __forceinline__ Spinor<T> receive_faces(const SapArgs& a, const void* faces, const ST& st, int blk, int r,
-                                                   const int y[4], const int n[4], int hf) {
+// ---- face contributions of the other colour.  A site lies on at most one face
+// per direction (block extents are at least 2): "up" (y_mu = b_mu - 1) takes the
+// block at +mu's projected spinor, multiplied here by the site's link, "down" the
+// block at -mu's, already multiplied by the sender.  The loads of both sites and
+// both directions of a thread are issued together at the start of a block, before
+// it waits for its staging copies, so that one memory latency passes for all of
+// them (four one after another took 8,000 of a block's 84,000 cycles).
+template <typename T>
+struct FaceIn {
+  Half<T> h;
+  T sgn;  // -1: up, +1: down, 0: not on a face in this direction
+};
+
+template <int MU, typename T>
+__device__ __forceinline__ FaceIn<T> face_fetch(const SapArgs& a, const void* faces, int blk, const int y[4],
+                                                const int n[4], bool on) {
   const Geom& g = a.g;
+  FaceIn<T> f;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.h.c[s][c] = {T(0), T(0)};
+  const bool up = y[MU] == g.b[MU] - 1, down = y[MU] == 0;
+  f.sgn = up ? T(-1) : (down ? T(1) : T(0));
+  if (on && (up || down)) {
+    const int nbk = up ? (n[MU] + 1 < g.nb[MU] ? blk + g.bstr[MU] : blk - (g.nb[MU] - 1) * g.bstr[MU])
+                       : (n[MU] > 0 ? blk - g.bstr[MU] : blk + (g.nb[MU] - 1) * g.bstr[MU]);
+    f.h = face_load<T>(a, faces, nbk, up ? 2 * MU : 2 * MU + 1, face_index(g, y, MU));
+  }
+  return f;
+}
+
+template <typename T>
+__device__ __forceinline__ void fetch_faces(const SapArgs& a, const void* faces, int blk, const int ye[4],
+                                            const int yo[4], const int n[4], int hf, FaceIn<T>& e0, FaceIn<T>& e1,
+                                            FaceIn<T>& o0, FaceIn<T>& o1) {
+  if (hf) {
+    e0 = face_fetch<2, T>(a, faces, blk, ye, n, a.faces_in);
+    e1 = face_fetch<3, T>(a, faces, blk, ye, n, a.faces_in);
+    o0 = face_fetch<2, T>(a, faces, blk, yo, n, a.faces_in);
+    o1 = face_fetch<3, T>(a, faces, blk, yo, n, a.faces_in);
+  } else {
+    e0 = face_fetch<0, T>(a, faces, blk, ye, n, a.faces_in);
+    e1 = face_fetch<1, T>(a, faces, blk, ye, n, a.faces_in);
+    o0 = face_fetch<0, T>(a, faces, blk, yo, n, a.faces_in);
+    o1 = face_fetch<1, T>(a, faces, blk, yo, n, a.faces_in);
+  }
+}
+
+// acc += the received contribution in direction MU
+template <int MU, typename T, typename ST>
+__device__ __forceinline__ void face_add(Spinor<T>& acc, const ST& st, int r, const FaceIn<T>& f) {
+  if (f.sgn == T(0)) return;
+  Half<T> w = f.h;
+  if (f.sgn < T(0)) w = umul(st.link(r, MU), f.h);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cpx<T> w0 = w.c[0][a], w1 = w.c[1][a];
+    acc.c[0][a] = acc.c[0][a] + w0;
+    acc.c[1][a] = acc.c[1][a] + w1;
+    if (MU == 0) {
+      fadd(acc.c[2][a], -f.sgn, w0);
+      fadd(acc.c[3][a], -f.sgn, w1);
+    } else if (MU == 1) {
+      fadd_i(acc.c[2][a], f.sgn, w1);
+      fadd_i(acc.c[3][a], f.sgn, w0);
+    } else if (MU == 2) {
+      fadd(acc.c[2][a], f.sgn, w1);
+      fadd(acc.c[3][a], -f.sgn, w0);
+    } else {
+      fadd_i(acc.c[2][a], f.sgn, w0);
+      fadd_i(acc.c[3][a], -f.sgn, w1);
+    }
+  }
+}
+
+// the contributions a thread fetched for one site, in its directions 2 hf and 2 hf + 1
+template <typename T, typename ST>
+__device__ __forceinline__ Spinor<T> face_sum(const ST& st, int r, const FaceIn<T>& f0, const FaceIn<T>& f1, int hf) {
   Spinor<T> acc;
   zero(acc);
-#pragma unroll 1
-  for (int m = 0; m < 2; ++m) {
-    const int mu = 2 * hf + m;
-    const SpinDir<T> d = spin_dir<T>(mu);
-    const int ymu = mu == 0 ? y[0] : (mu == 1 ? y[1] : (mu == 2 ? y[2] : y[3]));
-    const int nmu = mu == 0 ? n[0] : (mu == 1 ? n[1] : (mu == 2 ? n[2] : n[3]));
-    // up: from block + mu, U_mu(y) (1 - g) part, projected by the sender;
-    // down: from block - mu, U^+ (1 + g) part, multiplied by the sender
-    const bool up = ymu == g.b[mu] - 1, down = ymu == 0;
-    if (!up && !down) continue;
-    const int nbk = up ? (nmu + 1 < g.nb[mu] ? blk + g.bstr[mu] : blk - (g.nb[mu] - 1) * g.bstr[mu])
-                       : (nmu > 0 ? blk - g.bstr[mu] : blk + (g.nb[mu] - 1) * g.bstr[mu]);
-    const Half<T> h = face_load<T>(a, faces, nbk, up ? 2 * mu : 2 * mu + 1, face_index(g, y, mu));
-    if (up)
-      expand_add_rt<-1>(acc, umul(st.link(r, mu), h), T(1), d);
-    else
-      expand_add_rt<+1>(acc, h, T(1), d);
+  if (hf) {
+    face_add<2>(acc, st, r, f0);
+    face_add<3>(acc, st, r, f1);
+  } else {
+    face_add<0>(acc, st, r, f0);
+    face_add<1>(acc, st, r, f1);
   }
   return acc;
 }
 
-// write the face contributions of the correction chi at site (blk, r) for the
-// directions of this thread
+// write the face contribution of the correction chi at site (blk, r) in direction MU
+template <int MU, typename T, typename ST>
+__device__ __forceinline__ void send_face(const SapArgs& a, void* faces, const ST& st, int blk, int r, const int y[4],
+                                          const int n[4], const Spinor<T>& chi) {
+  const Geom& g = a.g;
+  const bool low = y[MU] == 0;  // to y = x - mu: 1/2 eta_mu(y) (1 - g) chi, projected
+  if (!low && y[MU] != g.b[MU] - 1) return;
+  const bool wrap = low ? n[MU] == 0 : n[MU] == g.nb[MU] - 1;
+  const T f = T(0.5) * (wrap ? bc_of<T>(g, MU) : T(1));
+  Half<T> h;
+  if (low)
+    h = project<MU, -1>(chi);
+  else  // to y = x + mu: 1/2 eta_mu(x) U_mu(x)^+ (1 + g) chi, projected
+    h = udmul(st.link(r, MU), project<MU, +1>(chi));
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h.c[s][c] = f * h.c[s][c];
+  face_store<T>(a, faces, blk, low ? 2 * MU : 2 * MU + 1, face_index(g, y, MU), h);
+}
+
 template <typename T, typename ST>
 __device__ __forceinline__ void send_faces(const SapArgs& a, void* faces, const ST& st, int blk, int r,
                                            const int y[4], const int n[4], const Spinor<T>& chi, int hf) {
-  const Geom& g = a.g;
-#pragma unroll 1
-  for (int m = 0; m < 2; ++m) {
-    const int mu = 2 * hf + m;
-    const SpinDir<T> d = spin_dir<T>(mu);
-    const int ymu = mu == 0 ? y[0] : (mu == 1 ? y[1] : (mu == 2 ? y[2] : y[3]));
-    const int nmu = mu == 0 ? n[0] : (mu == 1 ? n[1] : (mu == 2 ? n[2] : n[3]));
-    if (ymu == 0) {  // to y = x - mu: 1/2 eta_mu(y) (1 - g) chi, projected
-      const T f = T(0.5) * ((nmu == 0) ? bc_of<T>(g, mu) : T(1));
-      Half<T> h = project_rt<-1>(chi, d);
+  if (hf) {
+    send_face<2>(a, faces, st, blk, r, y, n, chi);
+    send_face<3>(a, faces, st, blk, r, y, n, chi);
+  } else {
+    send_face<0>(a, faces, st, blk, r, y, n, chi);
+    send_face<1>(a, faces, st, blk, r, y, n, chi);
+  }
+}
+
+// a spinor from the thread's own half and its partner's
+template <typename T>
+__device__ __forceinline__ Spinor<T> join_halves(const Half<T>& own, const Half<T>& other, int hf) {
+  Spinor<T> v;
 #pragma unroll
-      for (int s = 0; s < 2; ++s)
+  for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) h.c[s][c] = f * h.c[s][c];
-      face_store<T>(a, faces, blk, 2 * mu, face_index(g, y, mu), h);
+    for (int c = 0; c < 3; ++c) {
+      v.c[s][c] = hf ? other.c[s][c] : own.c[s][c];
+      v.c[2 + s][c] = hf ? own.c[s][c] : other.c[s][c];
     }
-    if (ymu == g.b[mu] - 1) {  // to y = x + mu: 1/2 eta_mu(x) U_mu(x)^+ (1 + g) chi, projected
-      const T f = T(0.5) * ((nmu == g.nb[mu] - 1) ? bc_of<T>(g, mu) : T(1));
-      Half<T> w = udmul(st.link(r, mu), project_rt<+1>(chi, d));
+  return v;
+}
+
+template <typename T>
+__device__ __forceinline__ T half_max(const Half<T>& h) {
+  T m = 0;
 #pragma unroll
-      for (int s = 0; s < 2; ++s)
+  for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) w.c[s][c] = f * w.c[s][c];
-      face_store<T>(a, faces, blk, 2 * mu + 1, face_index(g, y, mu), w);
+    for (int c = 0; c < 3; ++c) m = fmax(m, fmax(fabs(h.c[s][c].re), fabs(h.c[s][c].im)));
+  return m;
+}
+
+// store the owned half of a residual record; 16-bit records get the scale `m`, the
+// maximum over both halves (written by half 0)
+template <int P, typename T>
+__device__ __forceinline__ void rho_half_store(const FieldPtr& f, int Vb, int blk, int r, int hf, const Half<T>& h,
+                                               T m) {
+  if constexpr (P == P16 || P == PB16) {
+    typedef typename Storage<P>::real hr;
+    const float inv = m > 0.f ? 1.0f / m : 0.f;
+    uint32_t w[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      hr* q = reinterpret_cast<hr*>(&w[k]);
+      q[0] = from_f<P>(h.c[k / 3][k % 3].re * inv);
+      q[1] = from_f<P>(h.c[k / 3][k % 3].im * inv);
     }
+    uint4* d = (uint4*)f.data + (long long)blk * 3 * Vb + r;
+    if (hf == 0) {
+      d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+      *((uint2*)(d + Vb)) = make_uint2(w[4], w[5]);
+      f.norm[(long long)blk * Vb + r] = m;
+    } else {
+      *((uint2*)(d + Vb) + 1) = make_uint2(w[0], w[1]);
+      d[2 * (long long)Vb] = make_uint4(w[2], w[3], w[4], w[5]);
+    }
+  } else {
+    g_half_store<P, T>(f, Vb, blk, r, hf, h);
   }
 }
 
@@ -838,8 +967,16 @@ __host__ __device__ __forceinline__ int pairs_per_half(int Vbh) { return (Vbh + 
 // offsets become immediates, which frees registers), or 0 for any volume
 // TILED: the CTA solves a tile of right-hand sides (the loop below runs over
 // them); otherwise exactly one, right-hand side 0, and the loop folds away
+// Threads: the largest block whose fields fit in shared memory has 512 sites in
+// 16-bit form, 320 in FP32 and 144 in FP64 -- two threads per pair of sites, in
+// whole warps per half -- so the wider arithmetic gets more registers.
+template <int P>
+struct SapThreads {
+  static constexpr int most = P == P64 ? 192 : (P == P32 ? 320 : 512);
+};
+
 template <int P, typename T, int VB, bool TILED>
-__global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
+__global__ void __launch_bounds__(SapThreads<P>::most) sap_sweep_kernel(SapArgs a) {
   typedef typename StageFor<P>::type ST;
   constexpr bool kHalf = (P == P16 || P == PB16);
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -880,9 +1017,11 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
 
   // ---- stage the block's links and clover (once for the whole tile)
   if constexpr (kHalf) {
-    if (threadIdx.x == 0) mbar_init(bar, 1);
-    __syncthreads();  // every thread sees the initialised barrier before it waits on it
-    if (threadIdx.x < 32) stage_issue<P>(a, blk, (unsigned char*)s_r, (unsigned char*)st.base + 144 * Vb, bar);
+    if (threadIdx.x < 32) {  // (the others see the initialised barrier after the first __syncthreads below)
+      if (threadIdx.x == 0) mbar_init(bar, 1);
+      __syncwarp();
+      stage_issue<P>(a, blk, (unsigned char*)s_r, (unsigned char*)st.base + 144 * Vb, bar);
+    }
   } else {
     for (int r = threadIdx.x; r < Vb; r += blockDim.x) {
 #pragma unroll 1
@@ -949,9 +1088,18 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
     if (threadIdx.x >= 32 && threadIdx.x < 64)
       prefetch_late_reads<T, PsiPrec<P>::value>(a, rhs_faces(a, rr), rhs_psi(a, rr), blk, n);
 
-    // ---- residual of the two sites (own halves only: the pair's two threads
-    // read complementary halves)
+    // ---- what the block reads from memory, all asked for before the first wait:
+    // the faces (both sites, own directions), then the residual (own halves only:
+    // the pair's two threads read complementary halves).  A stored residual is 0 on
+    // odd sites (the block solve ends with it), so those are neither stored nor read.
+    FaceIn<T> fe0, fe1, fo0, fo1;
+    const bool faces_ahead = sizeof(T) == 4;  // (FP64 halves would not fit the registers)
+    if (faces_ahead) fetch_faces(a, rhs_faces(a, rr), blk, ye, yo, n, hf, fe0, fe1, fo0, fo1);
     Half<T> rho_e, rho_o;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) rho_o.c[s][c] = {T(0), T(0)};
     if (a.read_eta && a.io32) {
       const Half<float> de = g_half<P32, float>(rhs_eta(a, rr), Vb, blk, re, hf);
       const Half<float> dd = g_half<P32, float>(rhs_eta(a, rr), Vb, blk, ro, hf);
@@ -970,13 +1118,12 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
       rho_o = g_half<P64, T>(rhs_eta(a, rr), Vb, blk, ro, hf);
     } else if constexpr (kHalf) {
       rho_e = g_half16<P>(rhs_rho(a, rr), Vb, blk, re, hf);
-      rho_o = g_half16<P>(rhs_rho(a, rr), Vb, blk, ro, hf);
     } else {
       rho_e = g_half<P, T>(rhs_rho(a, rr), Vb, blk, re, hf);
-      rho_o = g_half<P, T>(rhs_rho(a, rr), Vb, blk, ro, hf);
     }
     if (!staged) {
       if constexpr (kHalf) {
+        __syncthreads();  // the barrier is initialised
         // every thread waits (bounded) for the staging copies; a time-out is made
         // block-uniform, recorded, and the block is skipped
         const bool ok = mbar_wait_bounded(bar, a.wait_cycles);
@@ -1001,14 +1148,21 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
     }
     if (TILED) __syncthreads();  // the previous right-hand side's last reads of r, t and the exchange buffer are done
     if (a.faces_in) {
-      rho_e = half_axpy(rho_e, pair_reduce_s(receive_faces<T>(a, rhs_faces(a, rr), st, blk, re, ye, n, hf), hf, i, np, s_x),
-                        T(1));
-      __syncthreads();
-      rho_o = half_axpy(rho_o, pair_reduce_s(receive_faces<T>(a, rhs_faces(a, rr), st, blk, ro, yo, n, hf), hf, i, np, s_x),
-                        T(1));
+      if (!faces_ahead) fetch_faces(a, rhs_faces(a, rr), blk, ye, yo, n, hf, fe0, fe1, fo0, fo1);
+      // both sites' partial sums change hands together: the part the partner owns
+      // goes to the partner's slots of the exchange buffer (even site) and of t
+      // (odd site), which only the partner writes afterwards
+      const Spinor<T> pe = face_sum(st, re, fe0, fe1, hf), po = face_sum(st, ro, fo0, fo1, hf);
+      s_half_store(s_x, np, i, 1 - hf, half_of(pe, 1 - hf));
+      if (act) s_half_store(s_t, ns, i, 1 - hf, half_of(po, 1 - hf));
+      pair_warps_sync(i);
+      rho_e = half_axpy(rho_e, half_axpy(half_of(pe, hf), s_half(s_x, np, i, hf), T(1)), T(1));
+      rho_o = half_axpy(rho_o, half_axpy(half_of(po, hf), s_half(s_t, ns, re, hf), T(1)), T(1));
     }
-    // etahat = rho_e - D_eo A_oo^-1 rho_o: first t = A_oo^-1 rho_o
-    if (act) s_half_store(s_t, ns, i, hf, clover_half(st, ro, hf, rho_o));
+    // etahat = rho_e - D_eo A_oo^-1 rho_o: first t = A_oo^-1 rho_o, which is also
+    // where chi_o starts
+    Half<T> chi_o = clover_half(st, ro, hf, rho_o);
+    if (act) s_half_store(s_t, ns, i, hf, chi_o);
     __syncthreads();
     Half<T> r = half_axpy(rho_e, block_hops<T>(st, ns, re, s_t, pkE, Vbh, hf, i, np, s_x), T(-1));
     Half<T> x;
@@ -1019,60 +1173,82 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
     if (act) s_half_store(s_r, ns, i, hf, r);
     __syncthreads();
 
-    // ---- MR on Dhat = A_ee - D_eo A_oo^-1 D_oe, x_e = 0, r = etahat.  Each
-    // step runs two phases through one code path: phase 0 (odd sites)
-    // t = A_oo^-1 D_oe r, phase 1 (even sites) p = A_ee r - D_eo t.
-#pragma unroll 1
-    for (int step = 0; step < 2 * a.nmr; ++step) {
-      const int ph = step & 1;
-      const int pk2[2] = {ph ? pkE[0] : pkO[0], ph ? pkE[1] : pkO[1]};
-      const Half<T> hq = block_hops<T>(st, ns, ph ? re : ro, ph ? s_t : s_r, pk2, ph ? Vbh : 0, hf, i, np, s_x);
-      const Half<T> cl = clover_half(st, ph ? re : ro, hf, ph ? r : hq);
-      if (ph == 0) {
-        if (act) s_half_store(s_t, ns, i, hf, cl);
-        __syncthreads();
-        continue;
-      }
-      const Half<T> p = half_axpy(cl, hq, T(-1));
-      T pr_re = 0, pr_im = 0, pp = 0;
-      if (act) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const cpx<T> v = p.c[s][c], w = r.c[s][c];
-            pr_re += v.re * w.re + v.im * w.im;
-            pr_im += v.re * w.im - v.im * w.re;
-            pp += v.re * v.re + v.im * v.im;
-          }
-      }
-      cta_sum3(pr_re, pr_im, pp, s_red);
+    if constexpr (kHalf) {
+      if (threadIdx.x >= 64 && threadIdx.x < 96) prefetch_next_block(a);
+    }
+
+    // ---- MR on Dhat = A_ee - D_eo A_oo^-1 D_oe from x_e = 0, r = etahat:
+    //   t = A_oo^-1 D_oe r;  p = A_ee r - D_eo t;  a = (p, r) / |p|^2;
+    //   x += a r;  r -= a p.
+    // Two things follow from linearity.  t is updated with r, t -= a A_oo^-1 D_oe p,
+    // so p itself goes to shared memory and the next hops start before a is known:
+    // a step needs two CTA-wide barriers and no wait for the sums (three and one
+    // before).  And A_oo^-1 D_oe x = sum a t, so the back substitution chi_o = A_oo^-1 (rho_o - D_oe x_e) is one
+    // multiply-add per step instead of one more pass of hops.  Each step runs two
+    // phases through one code path: phase 0 (odd sites) t, phase 1 (even sites) p.
+    // With the loads ahead and the L2 prefetch, a launch on 32^3 x 64 in 8x4x4x4
+    // blocks went from 0.551 to 0.497 ms, for 12 right-hand sides on 24^3 x 48 from
+    // 2.30 to 1.95 ms.
+    cpx<T> alpha = {T(0), T(0)};
+    auto advance = [&] {  // with a of the finished step: x, r, chi_o (s_r holds p, s_t holds t)
+      T pr_re, pr_im, pp;
+      sum3_get(pr_re, pr_im, pp, s_red);
       const T inv = pp > T(0) ? T(1) / pp : T(0);
-      const cpx<T> alpha = {pr_re * inv, pr_im * inv};
+      alpha = {pr_re * inv, pr_im * inv};
+      const Half<T> p = s_half(s_r, ns, re, hf), t = s_half(s_t, ns, re, hf);
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           x.c[s][c] = cmadd(alpha, r.c[s][c], x.c[s][c]);
-          r.c[s][c] = r.c[s][c] - cmul(alpha, p.c[s][c]);
+          r.c[s][c] = cmadd(-alpha, p.c[s][c], r.c[s][c]);
+          chi_o.c[s][c] = cmadd(-alpha, t.c[s][c], chi_o.c[s][c]);
         }
-      if (act) s_half_store(s_r, ns, i, hf, r);
+    };
+#pragma unroll 1
+    for (int step = 0; step < 2 * a.nmr; ++step) {
+      const int ph = step & 1;
+      if (ph == 0 && step > 0) advance();
+      const int pk2[2] = {ph ? pkE[0] : pkO[0], ph ? pkE[1] : pkO[1]};
+      const Half<T> hq = block_hops<T>(st, ns, ph ? re : ro, ph ? s_t : s_r, pk2, ph ? Vbh : 0, hf, i, np, s_x);
+      Half<T> cl = clover_half(st, ph ? re : ro, hf, ph ? r : hq);
+      if (ph == 0) {
+        if (step > 0) {
+          const Half<T> t = s_half(s_t, ns, re, hf);
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cl.c[s][c] = cmadd(-alpha, cl.c[s][c], t.c[s][c]);
+        }
+        if (act) s_half_store(s_t, ns, i, hf, cl);
+      } else {
+        const Half<T> p = half_axpy(cl, hq, T(-1));
+        T pr_re = 0, pr_im = 0, pp = 0;
+        if (act) {
+          half_dots(p, r, pr_re, pr_im, pp);
+          s_half_store(s_r, ns, i, hf, p);
+        }
+        sum3_put(pr_re, pr_im, pp, s_red);
+      }
       __syncthreads();
     }
-
-    // ---- chi_o = A_oo^-1 (rho_o - D_oe chi_e)
-    if (act) s_half_store(s_r, ns, i, hf, x);
-    __syncthreads();
-    const Half<T> chi_o =
-        clover_half(st, ro, hf, half_axpy(rho_o, block_hops<T>(st, ns, ro, s_r, pkO, 0, hf, i, np, s_x), T(-1)));
-    __syncthreads();
+    if (a.nmr > 0) advance();
 
     // ---- outputs: solution, block residual (r on even, 0 on odd), faces
     constexpr int PS = PsiPrec<P>::value;
     typedef typename std::conditional<PS == P64, double, float>::type TS;
-    const Spinor<T> x_full = pair_full_s(x, hf, i, np, s_x);
-    const Spinor<T> chio_full = pair_full_s(chi_o, hf, i, np, s_x);
-    const Spinor<T> r_full = pair_full_s(r, hf, i, np, s_x);
+    // what the partner needs: chi_o goes to t and chi_e to r (both read for the last
+    // time by their own threads above), the maximum of r to the exchange buffer, into
+    // the slot this thread read last
+    T r_max = half_max(r);
+    if (act) {
+      s_half_store(s_t, ns, i, hf, chi_o);
+      s_half_store(s_r, ns, i, hf, x);
+    }
+    T* s_m = s_x + Chunk<T>::R * ((12 / Chunk<T>::R) * (1 - hf) * np + i);
+    *s_m = r_max;
+    pair_warps_sync(i);
+    r_max = fmax(r_max, s_x[Chunk<T>::R * ((12 / Chunk<T>::R) * hf * np + i)]);
     if (act) {
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {
@@ -1099,12 +1275,7 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
           g_half_store<P64, TS>(rhs_out(a, rr), Vb, blk, rs, hf, v);  // widened on the integer pipes
         }
       }
-      if (a.write_rho && hf == 0) {
-        store_spinor<P, T>(rhs_rho(a, rr), Vb, blk, re, r_full);
-        Spinor<T> z;
-        zero(z);
-        store_spinor<P, T>(rhs_rho(a, rr), Vb, blk, ro, z);
-      }
+      if (a.write_rho) rho_half_store<P, T>(rhs_rho(a, rr), Vb, blk, re, hf, r, r_max);
       if (a.faces_out) {
         // the coordinates again (cheaper than keeping 12 registers through the MR steps)
         int n2[4], ye2[4], yo2[4];
@@ -1115,8 +1286,8 @@ __global__ void __launch_bounds__(512) sap_sweep_kernel(SapArgs a) {
           ye2[mu] = ycoord(pe, mu);
           yo2[mu] = ycoord(po, mu);
         }
-        send_faces<T>(a, rhs_faces(a, rr), st, blk, re, ye2, n2, x_full, hf);
-        send_faces<T>(a, rhs_faces(a, rr), st, blk, ro, yo2, n2, chio_full, hf);
+        send_faces<T>(a, rhs_faces(a, rr), st, blk, re, ye2, n2, join_halves(x, s_half(s_r, ns, i, 1 - hf), hf), hf);
+        send_faces<T>(a, rhs_faces(a, rr), st, blk, ro, yo2, n2, join_halves(chi_o, s_half(s_t, ns, i, 1 - hf), hf), hf);
       }
     }
   }
@@ -1224,6 +1395,16 @@ int sap_tile(qcd_ctx* c, int nr) {
   return rt;
 }
 
+// CTAs of a 16-bit sweep that run at the same time: by shared memory (228 KB per
+// SM, 1 KB of it taken per CTA) and by registers (128 for each of 512 threads)
+static int sap_wave(const qcd_ctx* c, int prec) {
+  if (prec != P16 && prec != PB16) return 1 << 30;
+  const size_t smem = sap_smem_bytes<P16, float>(c->g);
+  const int threads = 2 * pairs_per_half(c->g.Vbh);
+  const int by_mem = (int)((228 << 10) / (smem + 1024)), by_regs = 512 / threads;
+  return c->sms * (by_mem < by_regs ? (by_mem < 1 ? 1 : by_mem) : by_regs);
+}
+
 // psi = M_SAP eta (both FP64 or both FP32 fields) for every right-hand side of
 // B (fields V sites apart; B.mask skips right-hand sides); allocates nothing
 // once sap_prepare ran for prec and B.n
@@ -1254,6 +1435,7 @@ int sap_apply(qcd_ctx* c, SapWork& w, const Rec& eta64, const Rec& psi64, int nc
   a.err = (int*)(c->d_scalars + 128);
   a.wait_cycles = c->dbg_sap_wait_cycles;
   a.extra_tx = c->dbg_sap_extra_tx;
+  a.wave = sap_wave(c, prec);
   int off = 0;
   for (int mu = 0; mu < 4; ++mu) {
     a.fo[2 * mu] = off;
