@@ -6,7 +6,8 @@
 // complex numbers per element; the recursion of the mixed-precision scheme).
 // FP32 kernels accumulate in FP32 per thread; every CTA and grid sum is FP64.
 // Every reduction is deterministic: fixed grid, per-CTA partial sums in a
-// fixed order, then one warp per value sums the partials in index order.
+// fixed order, then the CTA that finishes last sums the partials, one warp per
+// value, in index order.
 #include "internal.h"
 
 namespace qcd {
@@ -96,38 +97,95 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// reduce M values per thread over the CTA (in FP64); thread j < M writes
-// part[blockIdx.x * M + j]
-template <int M, typename A>
-__device__ __forceinline__ void cta_reduce_store(A (&v)[M], double* part) {
-  __shared__ double sh[kBlasThreads / 32][M > 0 ? M : 1];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+// The sums of M values over a warp's lanes, M + 3 FP64 additions instead of 5 M
+// (one holds a quarter of an SM's FP64 unit for 64 cycles, and all CTAs reduce at
+// the same time): at every step the lanes of a pair split the values they still
+// hold, each adding the half it keeps.  write(j, total) is called by one lane for
+// each value.
+template <int C, int O, typename W>
+__device__ __forceinline__ void warp_sums_step(double* v, int idx, int limit, W write) {
+  const int l = threadIdx.x & 31;
+  if constexpr (O == 0) {
 #pragma unroll
-  for (int j = 0; j < M; ++j) {
-    double t = warp_sum((double)v[j]);
-    if (l == 0) sh[w][j] = t;
+    for (int e = 0; e < C; ++e)
+      if (idx + e < limit) write(idx + e, v[e]);
+  } else if constexpr (C == 1) {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+    if (l & O) limit = 0;  // the other lane of the pair writes
+    warp_sums_step<1, O / 2>(v, idx, limit, write);
+  } else {
+    constexpr int H = (C + 1) / 2;
+    const bool up = (l & O) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double a = v[i], b = i + H < C ? v[i + H] : 0.0;
+      const double send = up ? a : b;
+      v[i] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    // the upper lane holds values idx + H .. idx + C - 1, the lower idx .. idx + H - 1
+    warp_sums_step<H, O / 2>(v, up ? idx + H : idx, up ? limit : min(limit, idx + H), write);
   }
+}
+
+// Sum M values per thread over the grid (in FP64) and hand value j's total to
+// write(j, total): the CTAs' sums go to part (value j of CTA b at [j][b], after
+// the head, whose first word counts the CTAs that are done and wraps to 0), and
+// the last CTA adds them, one warp per value, lanes striding over the CTAs in
+// order.  A separate kernel for that took 8 to 11 us (its launch and one warp's
+// chain of loads), five times per iteration.
+template <int M, typename A, typename W>
+__device__ __forceinline__ void grid_reduce(A (&v)[M], double* part, W write) {
+  __shared__ double sh[kBlasThreads / 32][M > 0 ? M : 1];
+  __shared__ int last;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const unsigned nb = gridDim.x;
+  double* data = part + kPartHead;
+  double d0[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j) d0[j] = (double)v[j];
+  warp_sums_step<M, 16>(d0, 0, M, [&](int j, double t) { sh[w][j] = t; });
   __syncthreads();
   if (threadIdx.x < M) {
     double t = 0;
     for (int k = 0; k < kBlasThreads / 32; ++k) t += sh[k][threadIdx.x];
-    part[(long long)blockIdx.x * M + threadIdx.x] = t;
+    __stcg(data + (size_t)threadIdx.x * nb + blockIdx.x, t);
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc((unsigned*)part, nb - 1) == nb - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int j = w; j < M; j += kBlasThreads / 32) {
+    const double* d = data + (size_t)j * nb;
+    double t = 0;
+#pragma unroll 8
+    for (unsigned p = l; p < nb; p += 32) t += __ldcg(d + p);
+    t = warp_sum(t);
+    if (l == 0) write(j, t);
   }
 }
 
-__global__ void reduce_partials_kernel(const double* __restrict__ part, int nparts, int stride, int m, double* out,
-                                       BatchDev bd) {
-  // one warp per value, lanes stride over partials in a fixed order
+// out[j] = sum of value j's partials, one CTA per value (for kernels that leave
+// plain partial sums: the residuals and the HMC sums)
+static constexpr int kReduceThreads = 512;
+__global__ void __launch_bounds__(kReduceThreads)
+    reduce_partials_kernel(const double* __restrict__ part, int nparts, int stride, double* out, BatchDev bd) {
+  __shared__ double sh[kReduceThreads / 32];
   if (rhs_skipped(bd)) return;
   part += blockIdx.y * bd.ps;
   out += blockIdx.y * bd.ss;
-  const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int l = threadIdx.x & 31;
-  if (j >= m) return;
+  const int j = blockIdx.x, w = threadIdx.x >> 5, l = threadIdx.x & 31;
   double t = 0;
-  for (int p = l; p < nparts; p += 32) t += part[(long long)p * stride + j];
+#pragma unroll 8
+  for (int p = threadIdx.x; p < nparts; p += kReduceThreads) t += part[(long long)p * stride + j];
   t = warp_sum(t);
-  if (l == 0) out[j] = t;
+  if (l == 0) sh[w] = t;
+  __syncthreads();
+  if (w == 0) {
+    t = warp_sum(l < kReduceThreads / 32 ? sh[l] : 0.0);
+    if (l == 0) out[j] = t;
+  }
 }
 
 static BatchDev dev_of(const Batch& B, long long vs) { return BatchDev{vs, B.ss, B.ps, B.mask, B.k}; }
@@ -135,9 +193,7 @@ static BatchDev dev_of(const Batch& B, long long vs) { return BatchDev{vs, B.ss,
 // out[j] = sum_p partials[p * stride + j], j < m (per right-hand side of B)
 int reduce_partials(const double* partials, int nparts, int stride, int m, double* out, cudaStream_t s,
                     const Batch& B) {
-  const int warps = 8;
-  const dim3 grid((m + warps - 1) / warps, B.n);
-  reduce_partials_kernel<<<grid, 32 * warps, 0, s>>>(partials, nparts, stride, m, out, dev_of(B, 0));
+  reduce_partials_kernel<<<dim3(m, B.n), kReduceThreads, 0, s>>>(partials, nparts, stride, out, dev_of(B, 0));
   QCD_LAUNCHED();
   return QCD_OK;
 }
@@ -155,15 +211,17 @@ __device__ __forceinline__ bool second_pass_needed(const double* gs) {
 template <typename R, int K, int NORM>
 __global__ void __launch_bounds__(kBlasThreads)
     multidot_kernel(VecList<typename VecT<R>::type> vl, int k, const typename VecT<R>::type* __restrict__ w, long long n,
-                    const double* cond, double* part, BatchDev bd) {
+                    const double* cond, double* part, double* out, double* out_norm, BatchDev bd) {
   typedef typename VecT<R>::type E;
   if (rhs_skipped(bd)) return;
   const long long ro = blockIdx.y * bd.vs;
   w += ro;
   if (cond) cond += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
-  if (cond != nullptr && !second_pass_needed(cond)) {  // skipped: zero partial sums, no reduction
-    if (threadIdx.x < 2 * K + NORM) part[(long long)blockIdx.x * (2 * K + NORM) + threadIdx.x] = 0.0;
+  out += blockIdx.y * bd.ss;
+  if (NORM) out_norm += blockIdx.y * bd.ss;
+  if (cond != nullptr && !second_pass_needed(cond)) {  // skipped: zero coefficients
+    if (blockIdx.x == 0 && threadIdx.x < 2 * k) out[threadIdx.x] = 0.0;
     return;
   }
   R acc[2 * K + NORM];
@@ -176,7 +234,12 @@ __global__ void __launch_bounds__(kBlasThreads)
       if (j < k) dot_acc(__ldg(vl.v[j] + ro + i), b, acc[2 * j], acc[2 * j + 1]);
     if (NORM) nrm_acc(b, acc[2 * K]);
   }
-  cta_reduce_store<2 * K + NORM>(acc, part);
+  grid_reduce<2 * K + NORM>(acc, part, [&](int j, double t) {
+    if (NORM && j == 2 * K)
+      *out_norm = t;
+    else if (j < 2 * k)
+      out[j] = t;
+  });
 }
 
 // w -= sum_j c_j v_j; then out[j] = (v_j, w) (DOT = 1) or out = {|w|^2, (w, rho)} (DOT = 2)
@@ -184,7 +247,7 @@ template <typename R, int K, int DOT>
 __global__ void __launch_bounds__(kBlasThreads)
     axpy_dot_kernel(VecList<typename VecT<R>::type> vl, int k, const double* __restrict__ coef,
                     typename VecT<R>::type* __restrict__ w, const typename VecT<R>::type* __restrict__ rho, long long n,
-                    const double* cond, double* part, BatchDev bd) {
+                    const double* cond, double* part, double* out, BatchDev bd) {
   typedef typename VecT<R>::type E;
   constexpr int M = DOT == 1 ? 2 * K : 3;
   if (rhs_skipped(bd)) return;
@@ -194,7 +257,8 @@ __global__ void __launch_bounds__(kBlasThreads)
   coef += blockIdx.y * bd.ss;
   if (cond) cond += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
-  if (cond != nullptr && !second_pass_needed(cond)) return;  // block-uniform: no partials written
+  out += blockIdx.y * bd.ss;
+  if (cond != nullptr && !second_pass_needed(cond)) return;  // (nothing reads its results then)
   R acc[M];
 #pragma unroll
   for (int j = 0; j < M; ++j) acc[j] = 0;
@@ -224,7 +288,9 @@ __global__ void __launch_bounds__(kBlasThreads)
       dot_acc(b, r, acc[1], acc[2]);
     }
   }
-  cta_reduce_store<M>(acc, part);
+  grid_reduce<M>(acc, part, [&](int j, double t) {
+    if (DOT == 2 || j < 2 * k) out[j] = t;
+  });
 }
 
 // Final Gram-Schmidt coefficients of iteration k: gs = {|chi|^2 before,
@@ -236,7 +302,7 @@ template <typename R>
 __global__ void __launch_bounds__(kBlasThreads)
     normalise_update_kernel(typename VecT<R>::type* __restrict__ chi, typename VecT<R>::type* __restrict__ rho,
                             const double* __restrict__ gs, int two_pass, double* cr, long long n, double* part,
-                            BatchDev bd) {
+                            double* out, BatchDev bd) {
   typedef typename VecT<R>::type E;
   if (rhs_skipped(bd)) return;
   chi += blockIdx.y * bd.vs;
@@ -244,6 +310,7 @@ __global__ void __launch_bounds__(kBlasThreads)
   gs += blockIdx.y * bd.ss;
   cr += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
+  out += blockIdx.y * bd.ss;
   const double* co = (two_pass && second_pass_needed(gs)) ? gs + 4 : gs + 1;
   const double nrm2 = co[0];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -262,7 +329,7 @@ __global__ void __launch_bounds__(kBlasThreads)
     chi[i] = rscale(x, inv);
     nrm_acc(r, acc[0]);
   }
-  cta_reduce_store<1>(acc, part);
+  grid_reduce<1>(acc, part, [&](int, double t) { *out = t; });
 }
 
 // x += sum_j g_j phi_j (j < k, or j < bd.k[r] per right-hand side)
@@ -351,14 +418,15 @@ __global__ void __launch_bounds__(kBlasThreads)
 
 template <typename R>
 __global__ void __launch_bounds__(kBlasThreads)
-    norm2_kernel(const typename VecT<R>::type* __restrict__ v, long long n, double* part, BatchDev bd) {
+    norm2_kernel(const typename VecT<R>::type* __restrict__ v, long long n, double* part, double* out, BatchDev bd) {
   if (rhs_skipped(bd)) return;
   v += blockIdx.y * bd.vs;
   part += blockIdx.y * bd.ps;
+  out += blockIdx.y * bd.ss;
   R acc[1] = {0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     nrm_acc(__ldg(v + i), acc[0]);
-  cta_reduce_store<1>(acc, part);
+  grid_reduce<1>(acc, part, [&](int, double t) { *out = t; });
 }
 
 // y = g5 x on the internal FP64 layout [blk][12 components][Vb]: components 6..11 are spins 2, 3
@@ -437,26 +505,28 @@ __device__ __forceinline__ float4 df_csub(const float4& b, const dfacc& tr, cons
   return make_float4(re.hi, re.lo, im.hi, im.lo);
 }
 
-template <int M>
-__device__ __forceinline__ void df_reduce_store(const dfacc (&a)[M], double* part) {
+template <int M, typename W>
+__device__ __forceinline__ void df_grid_reduce(const dfacc (&a)[M], double* part, W write) {
   double v[M];
 #pragma unroll
   for (int j = 0; j < M; ++j) v[j] = acc_value(a[j]);
-  cta_reduce_store<M>(v, part);
+  grid_reduce<M>(v, part, write);
 }
 
 // out[j] = (v_j, w), j < k <= K; with NORM also |w|^2 (as multidot_kernel)
 template <int K, int NORM>
 __global__ void __launch_bounds__(kBlasThreads)
     df_multidot_kernel(VecList<float4> vl, int k, const float4* __restrict__ w, long long n, const double* cond,
-                       double* part, BatchDev bd) {
+                       double* part, double* out, double* out_norm, BatchDev bd) {
   if (rhs_skipped(bd)) return;
   const long long ro = blockIdx.y * bd.vs;
   w += ro;
   if (cond) cond += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
-  if (cond != nullptr && !second_pass_needed(cond)) {  // skipped: zero partial sums, no reduction
-    if (threadIdx.x < 2 * K + NORM) part[(long long)blockIdx.x * (2 * K + NORM) + threadIdx.x] = 0.0;
+  out += blockIdx.y * bd.ss;
+  if (NORM) out_norm += blockIdx.y * bd.ss;
+  if (cond != nullptr && !second_pass_needed(cond)) {  // skipped: zero coefficients
+    if (blockIdx.x == 0 && threadIdx.x < 2 * k) out[threadIdx.x] = 0.0;
     return;
   }
   dfacc acc[2 * K + NORM];
@@ -469,7 +539,12 @@ __global__ void __launch_bounds__(kBlasThreads)
       if (j < k) df_dot_acc(__ldg(vl.v[j] + ro + i), b, acc[2 * j], acc[2 * j + 1]);
     if (NORM) df_nrm_acc(b, acc[2 * K]);
   }
-  df_reduce_store<2 * K + NORM>(acc, part);
+  df_grid_reduce<2 * K + NORM>(acc, part, [&](int j, double t) {
+    if (NORM && j == 2 * K)
+      *out_norm = t;
+    else if (j < 2 * k)
+      out[j] = t;
+  });
 }
 
 // w -= sum_j c_j v_j; then {|w|^2, (w, rho)} (as axpy_dot_kernel with DOT = 2)
@@ -477,7 +552,7 @@ template <int K>
 __global__ void __launch_bounds__(kBlasThreads)
     df_axpy_norm_dot_kernel(VecList<float4> vl, int k, const double* __restrict__ coef, float4* __restrict__ w,
                             const float4* __restrict__ rho, long long n, const double* cond, double* part,
-                            BatchDev bd) {
+                            double* out, BatchDev bd) {
   if (rhs_skipped(bd)) return;
   const long long ro = blockIdx.y * bd.vs;
   w += ro;
@@ -485,7 +560,8 @@ __global__ void __launch_bounds__(kBlasThreads)
   coef += blockIdx.y * bd.ss;
   if (cond) cond += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
-  if (cond != nullptr && !second_pass_needed(cond)) return;  // block-uniform: no partials written
+  out += blockIdx.y * bd.ss;
+  if (cond != nullptr && !second_pass_needed(cond)) return;  // (nothing reads its results then)
   df cr[K], ci[K];
 #pragma unroll
   for (int j = 0; j < K; ++j) {
@@ -506,19 +582,20 @@ __global__ void __launch_bounds__(kBlasThreads)
     df_nrm_acc(b, acc[0]);
     df_dot_acc(b, __ldg(rho + i), acc[1], acc[2]);
   }
-  df_reduce_store<3>(acc, part);
+  df_grid_reduce<3>(acc, part, [&](int j, double t) { out[j] = t; });
 }
 
 // as normalise_update_kernel: chi /= |chi|; rho -= ((chi, rho) / |chi|^2) chi_unnormalised; |rho|^2
 __global__ void __launch_bounds__(kBlasThreads)
     df_normalise_update_kernel(float4* __restrict__ chi, float4* __restrict__ rho, const double* __restrict__ gs,
-                               int two_pass, double* cr, long long n, double* part, BatchDev bd) {
+                               int two_pass, double* cr, long long n, double* part, double* out, BatchDev bd) {
   if (rhs_skipped(bd)) return;
   chi += blockIdx.y * bd.vs;
   rho += blockIdx.y * bd.vs;
   gs += blockIdx.y * bd.ss;
   cr += blockIdx.y * bd.ss;
   part += blockIdx.y * bd.ps;
+  out += blockIdx.y * bd.ss;
   const double* co = (two_pass && second_pass_needed(gs)) ? gs + 4 : gs + 1;
   const double nrm2 = co[0];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -539,7 +616,7 @@ __global__ void __launch_bounds__(kBlasThreads)
     chi[i] = make_float4(xr.hi, xr.lo, xi.hi, xi.lo);
     df_nrm_acc(r, acc[0]);
   }
-  df_reduce_store<1>(acc, part);
+  df_grid_reduce<1>(acc, part, [&](int, double t) { *out = t; });
 }
 
 // x64 += sum_j g_j phi_j with double-float phi_j: the sum formed in
@@ -685,15 +762,14 @@ int blas_multidot(qcd_ctx* c, double* part, const R* const* v, int k, const R* w
   while (done < k) {
     const int kk = k - done < K ? k - done : K;
     const int norm = (d_norm != nullptr && done == 0) ? 1 : 0;
-    const int M = 2 * K + norm;
     auto vl = make_list<R>(v + done, kk);
     const E* w2 = (const E*)w;
     const dim3 g2(grid, B.n);
 #define MD(KK)                                                                           \
   if (norm)                                                                              \
-    multidot_kernel<R, KK, 1><<<g2, kBlasThreads, 0, s>>>(vl, kk, w2, n, cond, part, bd); \
+    multidot_kernel<R, KK, 1><<<g2, kBlasThreads, 0, s>>>(vl, kk, w2, n, cond, part, d_out + 2 * done, d_norm, bd); \
   else                                                                                   \
-    multidot_kernel<R, KK, 0><<<g2, kBlasThreads, 0, s>>>(vl, kk, w2, n, cond, part, bd);
+    multidot_kernel<R, KK, 0><<<g2, kBlasThreads, 0, s>>>(vl, kk, w2, n, cond, part, d_out + 2 * done, nullptr, bd);
     switch (K) {
       case 4: MD(4); break;
       case 8: MD(8); break;
@@ -702,8 +778,6 @@ int blas_multidot(qcd_ctx* c, double* part, const R* const* v, int k, const R* w
     }
 #undef MD
     QCD_LAUNCHED();
-    QCD_TRY(reduce_partials(part, (int)grid, M, 2 * kk, d_out + 2 * done, s, B));
-    if (norm) QCD_TRY(reduce_partials(part + 2 * K, (int)grid, M, 1, d_norm, s, B));
     done += kk;
   }
   return QCD_OK;
@@ -717,7 +791,6 @@ static int axpy_dot_impl(qcd_ctx* c, double* part, const R* const* v, int k, con
   const long long n = nel<R>(c);
   const unsigned grid = blas_grid(n);
   const int K = pick_k(k);
-  const int M = DOT == 1 ? 2 * K : 3;
   const double work = (cond ? 0.0 : 1.0) * B.n;  // conditional pass: counted as no work (see blas_multidot)
   ProfScope ps(c, QCD_KERNEL_BLAS, s, work * sizeof(E) * (double)n * (k + 2 + (DOT == 2)),
                work * 16.0 * c->V * 12 * k);
@@ -727,13 +800,13 @@ static int axpy_dot_impl(qcd_ctx* c, double* part, const R* const* v, int k, con
   const dim3 g2(grid, B.n);
   const BatchDev bd = dev_of(B, n);
   switch (K) {
-    case 4: axpy_dot_kernel<R, 4, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, bd); break;
-    case 8: axpy_dot_kernel<R, 8, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, bd); break;
-    case 16: axpy_dot_kernel<R, 16, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, bd); break;
-    default: axpy_dot_kernel<R, 32, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, bd); break;
+    case 4: axpy_dot_kernel<R, 4, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, d_out, bd); break;
+    case 8: axpy_dot_kernel<R, 8, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, d_out, bd); break;
+    case 16: axpy_dot_kernel<R, 16, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, d_out, bd); break;
+    default: axpy_dot_kernel<R, 32, DOT><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w2, r2, n, cond, part, d_out, bd); break;
   }
   QCD_LAUNCHED();
-  return reduce_partials(part, (int)grid, M, DOT == 1 ? 2 * k : 3, d_out, s, B);
+  return QCD_OK;
 }
 
 template <typename R>
@@ -754,9 +827,9 @@ int blas_axpy_norm_dot(qcd_ctx* c, double* part, const R* const* v, int k, const
     auto vl = make_list<R>(v, 0);
     ProfScope ps(c, QCD_KERNEL_BLAS, s, 2.0 * sizeof(E) * n * B.n, 8.0 * c->V * 12 * B.n);
     axpy_dot_kernel<R, 4, 2><<<dim3(grid, B.n), kBlasThreads, 0, s>>>(vl, 0, d_coef, (E*)w, (const E*)rho, n, cond,
-                                                                       part, dev_of(B, n));
+                                                                       part, d_out, dev_of(B, n));
     QCD_LAUNCHED();
-    return reduce_partials(part, (int)grid, 3, 3, d_out, s, B);
+    return QCD_OK;
   }
   return axpy_dot_impl<R, 2>(c, part, v, k, d_coef, w, rho, d_out, s, cond, B);
 }
@@ -770,10 +843,10 @@ int blas_normalise_update(qcd_ctx* c, double* part, R* chi, R* rho, const double
   {
     ProfScope ps(c, QCD_KERNEL_BLAS, s, 4.0 * sizeof(E) * n * B.n, 8.0 * c->V * 12 * B.n);
     normalise_update_kernel<R><<<dim3(grid, B.n), kBlasThreads, 0, s>>>((E*)chi, (E*)rho, d_gs, two_pass, d_cr, n,
-                                                                         part, dev_of(B, n));
+                                                                         part, d_out, dev_of(B, n));
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_out, s, B);
+  return QCD_OK;
 }
 
 template <typename R>
@@ -844,10 +917,10 @@ int blas_norm2(qcd_ctx* c, double* part, const R* v, double* d_out, cudaStream_t
   const unsigned grid = blas_grid(n);
   {
     ProfScope ps(c, QCD_KERNEL_BLAS, s, sizeof(E) * (double)n * B.n, 4.0 * c->V * 12 * B.n);
-    norm2_kernel<R><<<dim3(grid, B.n), kBlasThreads, 0, s>>>((const E*)v, n, part, dev_of(B, n));
+    norm2_kernel<R><<<dim3(grid, B.n), kBlasThreads, 0, s>>>((const E*)v, n, part, d_out, dev_of(B, n));
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_out, s, B);
+  return QCD_OK;
 }
 
 // x /= |x| with |x|^2 taken from the Gram-Schmidt results gs (pass 2 when it
@@ -876,7 +949,7 @@ int blas_gs_normalise(qcd_ctx* c, double* x, const double* d_gs, int two_pass, d
 __global__ void __launch_bounds__(kBlasThreads)
     cg_update_kernel(double2* __restrict__ x, double2* __restrict__ r, const double2* __restrict__ p,
                      const double2* __restrict__ q, const double* __restrict__ rr, const double* __restrict__ tt,
-                     long long n, double* part) {
+                     long long n, double* part, double* out) {
   const double alpha = *tt > 0 ? *rr / *tt : 0.0;
   double acc[1] = {0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -890,7 +963,7 @@ __global__ void __launch_bounds__(kBlasThreads)
     r[i] = ri;
     nrm_acc(ri, acc[0]);
   }
-  cta_reduce_store<1>(acc, part);
+  grid_reduce<1>(acc, part, [&](int, double t) { *out = t; });
 }
 
 // p = r + (rr_new / rr) p
@@ -914,10 +987,10 @@ int blas_cg_update(qcd_ctx* c, double* part, double* x, double* r, const double*
   {
     ProfScope ps(c, QCD_KERNEL_BLAS, s, 96.0 * n, 10.0 * n);
     cg_update_kernel<<<grid, kBlasThreads, 0, s>>>((double2*)x, (double2*)r, (const double2*)p, (const double2*)q,
-                                                    d_rr, d_tt, n, part);
+                                                    d_rr, d_tt, n, part, d_rr_new);
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_rr_new, s);
+  return QCD_OK;
 }
 
 int blas_cg_direction(qcd_ctx* c, double* p, const double* r, const double* d_rr_new, const double* d_rr,
@@ -965,13 +1038,12 @@ int blas_df_multidot(qcd_ctx* c, double* part, const float4* const* v, int k, co
   while (done < k) {
     const int kk = k - done < K ? k - done : K;
     const int norm = (d_norm != nullptr && done == 0) ? 1 : 0;
-    const int M = 2 * K + norm;
     auto vl = make_df_list(v + done, kk);
 #define MD(KK)                                                                        \
   if (norm)                                                                           \
-    df_multidot_kernel<KK, 1><<<g2, kBlasThreads, 0, s>>>(vl, kk, w, n, cond, part, bd); \
+    df_multidot_kernel<KK, 1><<<g2, kBlasThreads, 0, s>>>(vl, kk, w, n, cond, part, d_out + 2 * done, d_norm, bd); \
   else                                                                                \
-    df_multidot_kernel<KK, 0><<<g2, kBlasThreads, 0, s>>>(vl, kk, w, n, cond, part, bd);
+    df_multidot_kernel<KK, 0><<<g2, kBlasThreads, 0, s>>>(vl, kk, w, n, cond, part, d_out + 2 * done, nullptr, bd);
     switch (K) {
       case 4: MD(4); break;
       case 8: MD(8); break;
@@ -979,8 +1051,6 @@ int blas_df_multidot(qcd_ctx* c, double* part, const float4* const* v, int k, co
     }
 #undef MD
     QCD_LAUNCHED();
-    QCD_TRY(reduce_partials(part, (int)grid, M, 2 * kk, d_out + 2 * done, s, B));
-    if (norm) QCD_TRY(reduce_partials(part + 2 * K, (int)grid, M, 1, d_norm, s, B));
     done += kk;
   }
   return QCD_OK;
@@ -998,13 +1068,13 @@ int blas_df_axpy_norm_dot(qcd_ctx* c, double* part, const float4* const* v, int 
   const dim3 g2(grid, B.n);
   const BatchDev bd = dev_of(B, n);
   switch (K) {
-    case 4: df_axpy_norm_dot_kernel<4><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, bd); break;
-    case 8: df_axpy_norm_dot_kernel<8><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, bd); break;
-    case 16: df_axpy_norm_dot_kernel<16><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, bd); break;
-    default: df_axpy_norm_dot_kernel<32><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, bd); break;
+    case 4: df_axpy_norm_dot_kernel<4><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
+    case 8: df_axpy_norm_dot_kernel<8><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
+    case 16: df_axpy_norm_dot_kernel<16><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
+    default: df_axpy_norm_dot_kernel<32><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
   }
   QCD_LAUNCHED();
-  return reduce_partials(part, (int)grid, 3, 3, d_out, s, B);
+  return QCD_OK;
 }
 
 int blas_df_normalise_update(qcd_ctx* c, double* part, float4* chi, float4* rho, const double* d_gs, int two_pass,
@@ -1014,10 +1084,10 @@ int blas_df_normalise_update(qcd_ctx* c, double* part, float4* chi, float4* rho,
   {
     ProfScope ps(c, QCD_KERNEL_BLAS, s, 64.0 * n * B.n, 8.0 * c->V * 12 * B.n);
     df_normalise_update_kernel<<<dim3(grid, B.n), kBlasThreads, 0, s>>>(chi, rho, d_gs, two_pass, d_cr, n, part,
-                                                                         dev_of(B, n));
+                                                                         d_out, dev_of(B, n));
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_out, s, B);
+  return QCD_OK;
 }
 
 int blas_df_update(qcd_ctx* c, const float4* const* phi, int k, const double* d_gamma, double* x, cudaStream_t s,

@@ -29,14 +29,7 @@ static int cg_prepare(qcd_ctx* c, Workspace& w, size_t nvec = 4) {
     w.cgv.emplace_back();
     QCD_TRY(rec_alloc(w.cgv.back(), P64, 24, c->V));
   }
-  if (!w.d_part) {
-    if (cudaMalloc(&w.d_part, sizeof(double) * partials_for(c->V)) != cudaSuccess) {
-      cudaGetLastError();
-      w.d_part = nullptr;
-      return QCD_ERR_NOMEM;
-    }
-    w.ps = (long long)partials_for(c->V);
-  }
+  if (!w.d_part) QCD_TRY(partials_alloc(c->V, 1, &w.d_part, &w.ps));
   if (!w.d_cg) QCD_CUDA(cudaMalloc(&w.d_cg, sizeof(double) * 8));
   if (!w.h_cg) QCD_CUDA(cudaMallocHost(&w.h_cg, sizeof(double) * 8));
   return QCD_OK;

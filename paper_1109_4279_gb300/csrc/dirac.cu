@@ -925,10 +925,10 @@ int residual64(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec& 
     ProfScope ps(c, QCD_KERNEL_RESIDUAL, s, (bytes_per_site(P64) + 192) * (double)c->V * B.n,
                  1848.0 * (double)c->V * B.n);
     residual64_kernel<<<dim3(grid, B.n), 256, 0, s>>>(c->g, c->U[P64], c->A[P64].ptr(), b.ptr(), x.ptr(), r.ptr(),
-                                                       part, B.ps, B.mask);
+                                                       part + kPartHead, B.ps, B.mask);
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_norm2, s, B);
+  return reduce_partials(part + kPartHead, (int)grid, 1, 1, d_norm2, s, B);
 }
 
 int residual_df(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec& r, const Rec& tmp, double* d_norm2,
@@ -944,10 +944,10 @@ int residual_df(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec&
     ProfScope ps(c, QCD_KERNEL_RESIDUAL, s, (bytes_per_site(P64) + 192) * (double)c->V * B.n,
                  1848.0 * (double)c->V * B.n);
     residual_df_kernel<<<dim3(grid, B.n), kDfThreads, 0, s>>>(c->g, (const float4*)c->U[PDF], c->A[PDF].ptr(), b.ptr(),
-                                                        tmp.ptr(), r.ptr(), part, B.ps, B.mask);
+                                                        tmp.ptr(), r.ptr(), part + kPartHead, B.ps, B.mask);
     QCD_LAUNCHED();
   }
-  return reduce_partials(part, (int)grid, 1, 1, d_norm2, s, B);
+  return reduce_partials(part + kPartHead, (int)grid, 1, 1, d_norm2, s, B);
 }
 
 // ------------------------------------------------------------------------

@@ -45,6 +45,10 @@ inline int chunks(int prec, int nreal) {
 // two CTAs of four fill an SM's gaps better than one of eight
 static constexpr int kDfThreads = 128;
 
+// doubles at the start of every right-hand side's partial sums; the first word is
+// the count of finished CTAs, 0 between kernels
+static constexpr int kPartHead = 4;
+
 // a device field of N-real records per site in one precision
 struct Rec {
   int prec = -1;
@@ -348,6 +352,8 @@ int reduce_partials(const double* partials, int nparts, int stride, int m, doubl
 
 // ---- solver.cu
 size_t partials_for(long long V);
+// allocate nr right-hand sides' partial sums (*ps doubles each), their heads cleared
+int partials_alloc(long long V, int nr, double** part, long long* ps);
 // allocate the solver fields and scalars of nr right-hand sides (a change of
 // nr reallocates everything)
 int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream_t s, int nr = 1);

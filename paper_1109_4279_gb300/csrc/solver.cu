@@ -43,7 +43,21 @@ namespace qcd {
 size_t partials_for(long long V) {
   const size_t blas = (size_t)152 * 8 * 65;     // largest BLAS grid x widest record
   const size_t resid = (size_t)(V + kDfThreads - 1) / kDfThreads;  // one partial per residual CTA
-  return blas > resid ? blas : resid;
+  return kPartHead + (blas > resid ? blas : resid);
+}
+
+int partials_alloc(long long V, int nr, double** part, long long* ps) {
+  const size_t n = partials_for(V);
+  if (cudaMalloc(part, sizeof(double) * n * nr) != cudaSuccess) {
+    cudaGetLastError();
+    *part = nullptr;
+    return QCD_ERR_NOMEM;
+  }
+  *ps = (long long)n;
+  // (the solver's streams do not wait for the default stream by themselves)
+  QCD_CUDA(cudaMemset2DAsync(*part, sizeof(double) * n, 0, sizeof(double) * kPartHead, nr, nullptr));
+  QCD_CUDA(cudaStreamSynchronize(nullptr));
+  return QCD_OK;
 }
 
 static void graphs_clear(Workspace& w) {
@@ -123,14 +137,7 @@ int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream
     w.pprec = pprec;
   }
   if (!w.rho.data) QCD_TRY(rec_alloc(w.rho, rprec, 24, Vn));
-  if (!w.d_part) {
-    w.ps = (long long)partials_for(c->V);
-    if (cudaMalloc(&w.d_part, sizeof(double) * w.ps * nr) != cudaSuccess) {
-      cudaGetLastError();
-      w.d_part = nullptr;
-      return QCD_ERR_NOMEM;
-    }
-  }
+  if (!w.d_part) QCD_TRY(partials_alloc(c->V, nr, &w.d_part, &w.ps));
   if (nkv > w.nkv) {
     graphs_clear(w);
     for (int k = w.nkv; k < nkv; ++k) {
