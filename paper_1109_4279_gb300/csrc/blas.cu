@@ -480,37 +480,51 @@ __global__ void backsub_kernel(const double* a1, const double* a2, const double*
 // faster.  Per-thread sums go to FP64 for the CTA and grid reductions.
 // ------------------------------------------------------------------------
 
-// (re, im) += conj(a) b
-__device__ __forceinline__ void df_dot_acc(const float4& a, const float4& b, dfacc& re, dfacc& im) {
-  acc_prod(re, a.x, a.y, b.x, b.y);
-  acc_prod(re, a.z, a.w, b.z, b.w);
-  acc_prod(im, a.x, a.y, b.z, b.w);
-  acc_prod(im, -a.z, -a.w, b.x, b.y);
-}
-__device__ __forceinline__ void df_nrm_acc(const float4& b, dfacc& n) {
-  acc_prod(n, b.x, b.y, b.x, b.y);
-  acc_prod(n, b.z, b.w, b.z, b.w);
-}
-// t = (cr + i ci) a accumulated into (tr, ti)
-__device__ __forceinline__ void df_cmul_acc(df cr, df ci, const float4& a, dfacc& tr, dfacc& ti) {
-  acc_prod(tr, cr.hi, cr.lo, a.x, a.y);
-  acc_prod(tr, -ci.hi, -ci.lo, a.z, a.w);
-  acc_prod(ti, cr.hi, cr.lo, a.z, a.w);
-  acc_prod(ti, ci.hi, ci.lo, a.x, a.y);
-}
-// b - (tr, ti) as a double-float complex element
-__device__ __forceinline__ float4 df_csub(const float4& b, const dfacc& tr, const dfacc& ti) {
-  const df re = df_add(df{b.x, b.y}, df_neg(acc_df(tr)));
-  const df im = df_add(df{b.z, b.w}, df_neg(acc_df(ti)));
-  return make_float4(re.hi, re.lo, im.hi, im.lo);
+// The two parts of a complex sum are the lanes of packed instructions: half the
+// issue slots of the scalar form.
+
+// Elements per thread and loop pass, all of whose loads are issued before the first
+// product; one element at a time left the memory idle (32^3 x 64, four vectors
+// dotted: 425 -> 306 us = 6.6 TB/s, subtracted: 540 -> 440 us).  More would cost the
+// warps that hide the arithmetic: eight vectors subtracted took 641 us with one
+// element and 784 us with two.
+constexpr int df_dot_unroll(int K) { return K <= 2 ? 4 : (K <= 8 ? 2 : 1); }
+constexpr int df_axpy_unroll(int K) { return K <= 4 ? 2 : 1; }
+__device__ __forceinline__ float4 ldg_if(bool on, const float4* p) {
+  return on ? __ldg(p) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-template <int M, typename W>
-__device__ __forceinline__ void df_grid_reduce(const dfacc (&a)[M], double* part, W write) {
-  double v[M];
-#pragma unroll
-  for (int j = 0; j < M; ++j) v[j] = acc_value(a[j]);
-  grid_reduce<M>(v, part, write);
+// what of b enters the products: (re, im) and the rotated (im, -re)
+struct DfElem {
+  df2 v, r;
+  __device__ __forceinline__ explicit DfElem(const float4& b)
+      : v{make_float2(b.x, b.z), make_float2(b.y, b.w)}, r{make_float2(b.z, -b.x), make_float2(b.w, -b.y)} {}
+};
+// (re, im) += conj(a) b
+__device__ __forceinline__ void df_dot_acc(const float4& a, const DfElem& b, acc2& s) {
+  acc2_prod<true>(s, bc2(a.x), bc2(a.y), b.v.hi, b.v.lo);
+  acc2_prod<true>(s, bc2(a.z), bc2(a.w), b.r.hi, b.r.lo);
+}
+// the squares of both parts, one per lane
+__device__ __forceinline__ void df_nrm_acc(const float4& b, acc2& n) {
+  const float2 h = make_float2(b.x, b.z), l = make_float2(b.y, b.w);
+  acc2_prod<true>(n, h, l, h, l);
+}
+// (tr, ti) += c a for the double-float coefficient c; LO: a has low parts
+template <bool LO>
+__device__ __forceinline__ void df_cmul_acc(df cr, df ci, float4 a, acc2& t) {
+  acc2_prod<LO>(t, bc2(cr.hi), bc2(cr.lo), make_float2(a.x, a.z), make_float2(a.y, a.w));
+  acc2_prod<LO>(t, bc2(ci.hi), bc2(ci.lo), make_float2(-a.z, a.x), make_float2(-a.w, a.y));
+}
+__device__ __forceinline__ double acc_value(const acc2& a, int part) {
+  return part ? f32_to_f64(a.s.y) + f32_to_f64(a.c.y) : f32_to_f64(a.s.x) + f32_to_f64(a.c.x);
+}
+__device__ __forceinline__ acc2 acc2_zero() { return acc2{bc2(0.f), bc2(0.f)}; }
+// b - t as a double-float complex element
+__device__ __forceinline__ float4 df_csub(const float4& b, const acc2& t) {
+  const df re = df_add(df{b.x, b.y}, df_neg(two_sum(t.s.x, t.c.x)));
+  const df im = df_add(df{b.z, b.w}, df_neg(two_sum(t.s.y, t.c.y)));
+  return make_float4(re.hi, re.lo, im.hi, im.lo);
 }
 
 // out[j] = (v_j, w), j < k <= K; with NORM also |w|^2 (as multidot_kernel)
@@ -529,17 +543,35 @@ __global__ void __launch_bounds__(kBlasThreads)
     if (blockIdx.x == 0 && threadIdx.x < 2 * k) out[threadIdx.x] = 0.0;
     return;
   }
-  dfacc acc[2 * K + NORM];
+  acc2 acc[K + NORM];
 #pragma unroll
-  for (int j = 0; j < 2 * K + NORM; ++j) acc[j] = {0.f, 0.f};
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float4 b = __ldg(w + i);
+  for (int j = 0; j < K + NORM; ++j) acc[j] = acc2_zero();
+  constexpr int U = df_dot_unroll(K);
+  const long long st = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += U * st) {
+    float4 b[U], x[U][K];
 #pragma unroll
-    for (int j = 0; j < K; ++j)
-      if (j < k) df_dot_acc(__ldg(vl.v[j] + ro + i), b, acc[2 * j], acc[2 * j + 1]);
-    if (NORM) df_nrm_acc(b, acc[2 * K]);
+    for (int u = 0; u < U; ++u) {
+      const bool on = i + u * st < n;
+      b[u] = ldg_if(on, w + i + u * st);
+#pragma unroll
+      for (int j = 0; j < K; ++j)
+        if (j < k) x[u][j] = ldg_if(on, vl.v[j] + ro + i + u * st);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const DfElem e(b[u]);
+#pragma unroll
+      for (int j = 0; j < K; ++j)
+        if (j < k) df_dot_acc(x[u][j], e, acc[j]);
+      if (NORM) df_nrm_acc(b[u], acc[K]);
+    }
   }
-  df_grid_reduce<2 * K + NORM>(acc, part, [&](int j, double t) {
+  double v[2 * K + NORM];
+#pragma unroll
+  for (int j = 0; j < 2 * K; ++j) v[j] = acc_value(acc[j >> 1], j & 1);
+  if (NORM) v[2 * K] = acc_value(acc[K], 0) + acc_value(acc[K], 1);
+  grid_reduce<2 * K + NORM>(v, part, [&](int j, double t) {
     if (NORM && j == 2 * K)
       *out_norm = t;
     else if (j < 2 * k)
@@ -568,21 +600,36 @@ __global__ void __launch_bounds__(kBlasThreads)
     cr[j] = j < k ? df_from_f64(coef[2 * j]) : df{0.f, 0.f};
     ci[j] = j < k ? df_from_f64(coef[2 * j + 1]) : df{0.f, 0.f};
   }
-  dfacc acc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    float4 b = w[i];
-    if (k > 0) {
-      dfacc tr = {0.f, 0.f}, ti = {0.f, 0.f};
+  acc2 nrm = acc2_zero(), dot = acc2_zero();
+  constexpr int U = df_axpy_unroll(K);
+  const long long st = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += U * st) {
+    float4 b[U], r[U], x[U][K];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool on = i + u * st < n;
+      b[u] = on ? w[i + u * st] : make_float4(0.f, 0.f, 0.f, 0.f);
+      r[u] = ldg_if(on, rho + i + u * st);
 #pragma unroll
       for (int j = 0; j < K; ++j)
-        if (j < k) df_cmul_acc(cr[j], ci[j], __ldg(vl.v[j] + ro + i), tr, ti);
-      b = df_csub(b, tr, ti);
-      w[i] = b;
+        if (j < k) x[u][j] = ldg_if(on, vl.v[j] + ro + i + u * st);
     }
-    df_nrm_acc(b, acc[0]);
-    df_dot_acc(b, __ldg(rho + i), acc[1], acc[2]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k > 0) {
+        acc2 t = acc2_zero();
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+          if (j < k) df_cmul_acc<true>(cr[j], ci[j], x[u][j], t);
+        b[u] = df_csub(b[u], t);
+        if (i + u * st < n) w[i + u * st] = b[u];
+      }
+      df_nrm_acc(b[u], nrm);
+      df_dot_acc(b[u], DfElem(r[u]), dot);
+    }
   }
-  df_grid_reduce<3>(acc, part, [&](int j, double t) { out[j] = t; });
+  double v[3] = {acc_value(nrm, 0) + acc_value(nrm, 1), acc_value(dot, 0), acc_value(dot, 1)};
+  grid_reduce<3>(v, part, [&](int j, double t) { out[j] = t; });
 }
 
 // as normalise_update_kernel: chi /= |chi|; rho -= ((chi, rho) / |chi|^2) chi_unnormalised; |rho|^2
@@ -605,18 +652,31 @@ __global__ void __launch_bounds__(kBlasThreads)
   }
   const df inv = df_from_f64(nrm2 > 0 ? 1.0 / sqrt(nrm2) : 0.0);
   const df cre = df_from_f64(nrm2 > 0 ? co[1] / nrm2 : 0.0), cim = df_from_f64(nrm2 > 0 ? co[2] / nrm2 : 0.0);
-  dfacc acc[1] = {{0.f, 0.f}};
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float4 x = chi[i];
-    dfacc tr = {0.f, 0.f}, ti = {0.f, 0.f};
-    df_cmul_acc(cre, cim, x, tr, ti);
-    const float4 r = df_csub(rho[i], tr, ti);
-    rho[i] = r;
-    const df xr = df_mul(df{x.x, x.y}, inv), xi = df_mul(df{x.z, x.w}, inv);
-    chi[i] = make_float4(xr.hi, xr.lo, xi.hi, xi.lo);
-    df_nrm_acc(r, acc[0]);
+  acc2 nrm = acc2_zero();
+  constexpr int U = 2;
+  const long long st = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += U * st) {
+    float4 x[U], r[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u == 0 || i + u * st < n) {
+        x[u] = chi[i + u * st];
+        r[u] = rho[i + u * st];
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u == 0 || i + u * st < n) {
+        acc2 t = acc2_zero();
+        df_cmul_acc<true>(cre, cim, x[u], t);
+        r[u] = df_csub(r[u], t);
+        rho[i + u * st] = r[u];
+        const df xr = df_mul(df{x[u].x, x[u].y}, inv), xi = df_mul(df{x[u].z, x[u].w}, inv);
+        chi[i + u * st] = make_float4(xr.hi, xr.lo, xi.hi, xi.lo);
+        df_nrm_acc(r[u], nrm);
+      }
   }
-  df_grid_reduce<1>(acc, part, [&](int, double t) { *out = t; });
+  double v[1] = {acc_value(nrm, 0) + acc_value(nrm, 1)};
+  grid_reduce<1>(v, part, [&](int, double t) { *out = t; });
 }
 
 // x64 += sum_j g_j phi_j with double-float phi_j: the sum formed in
@@ -638,13 +698,13 @@ __global__ void __launch_bounds__(kBlasThreads)
     gi[j] = j < k ? df_from_f64(gam[2 * j + 1]) : df{0.f, 0.f};
   }
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    dfacc tr = {0.f, 0.f}, ti = {0.f, 0.f};
+    double2 v = x[i];
+    acc2 t = acc2_zero();
 #pragma unroll
     for (int j = 0; j < K; ++j)
-      if (j < k) df_cmul_acc(gr[j], gi[j], __ldg(vl.v[j] + ro + i), tr, ti);
-    double2 v = x[i];
-    v.x += acc_value(tr);
-    v.y += acc_value(ti);
+      if (j < k) df_cmul_acc<true>(gr[j], gi[j], __ldg(vl.v[j] + ro + i), t);
+    v.x += acc_value(t, 0);
+    v.y += acc_value(t, 1);
     x[i] = v;
   }
 }
@@ -676,25 +736,26 @@ __global__ void __launch_bounds__(kBlasThreads)
     const int r = (int)(m - t * Vb), cc = (int)(t % 6);
     const long long blk = t / 6;
     const long long i0 = (blk * 12 + 2 * cc) * Vb + r;
-    dfacc tr0 = {0.f, 0.f}, ti0 = {0.f, 0.f}, tr1 = {0.f, 0.f}, ti1 = {0.f, 0.f};
+    acc2 t0 = acc2_zero(), t1 = acc2_zero();
+    double2 v = x[i0];
+    const double2 v1 = x[i0 + Vb];
 #pragma unroll
     for (int j = 0; j < K; ++j)
       if (j < k) {
         const float4 p = __ldg(vl.v[j] + ro + m);
-        df_cmul_acc(gr[j], gi[j], make_float4(p.x, 0.f, p.y, 0.f), tr0, ti0);
-        df_cmul_acc(gr[j], gi[j], make_float4(p.z, 0.f, p.w, 0.f), tr1, ti1);
+        df_cmul_acc<false>(gr[j], gi[j], make_float4(p.x, 0.f, p.y, 0.f), t0);
+        df_cmul_acc<false>(gr[j], gi[j], make_float4(p.z, 0.f, p.w, 0.f), t1);
       }
-    double2 v = x[i0];
-    v.x += acc_value(tr0);
-    v.y += acc_value(ti0);
+    v.x += acc_value(t0, 0);
+    v.y += acc_value(t0, 1);
     x[i0] = v;
     if (xs) {  // the updated x's double-float split too (same element order)
       const df a = df_from_f64(v.x), b = df_from_f64(v.y);
       xs[i0] = make_float4(a.hi, a.lo, b.hi, b.lo);
     }
-    v = x[i0 + Vb];
-    v.x += acc_value(tr1);
-    v.y += acc_value(ti1);
+    v = v1;
+    v.x += acc_value(t1, 0);
+    v.y += acc_value(t1, 1);
     x[i0 + Vb] = v;
     if (xs) {
       const df a = df_from_f64(v.x), b = df_from_f64(v.y);
@@ -1031,7 +1092,7 @@ int blas_df_multidot(qcd_ctx* c, double* part, const float4* const* v, int k, co
   const unsigned grid = blas_grid(n);
   const double work = (cond ? 0.0 : 1.0) * B.n;
   ProfScope ps(c, QCD_KERNEL_BLAS, s, work * 16.0 * (double)n * (k + 1), work * 8.0 * c->V * 12 * k);
-  const int K = pick_k(k) > 16 ? 16 : pick_k(k);
+  const int K = k <= 2 ? 2 : (pick_k(k) > 16 ? 16 : pick_k(k));
   const BatchDev bd = dev_of(B, n);
   const dim3 g2(grid, B.n);
   int done = 0;
@@ -1045,6 +1106,7 @@ int blas_df_multidot(qcd_ctx* c, double* part, const float4* const* v, int k, co
   else                                                                                \
     df_multidot_kernel<KK, 0><<<g2, kBlasThreads, 0, s>>>(vl, kk, w, n, cond, part, d_out + 2 * done, nullptr, bd);
     switch (K) {
+      case 2: MD(2); break;
       case 4: MD(4); break;
       case 8: MD(8); break;
       default: MD(16); break;
@@ -1061,13 +1123,14 @@ int blas_df_axpy_norm_dot(qcd_ctx* c, double* part, const float4* const* v, int 
   if (k > 32) return QCD_ERR_UNSUPPORTED;
   const long long n = c->V * 12;
   const unsigned grid = blas_grid(n);
-  const int K = k <= 4 ? 4 : (k <= 8 ? 8 : (k <= 16 ? 16 : 32));
+  const int K = k <= 1 ? 1 : (k <= 4 ? 4 : (k <= 8 ? 8 : (k <= 16 ? 16 : 32)));
   const double work = (cond ? 0.0 : 1.0) * B.n;
   ProfScope ps(c, QCD_KERNEL_BLAS, s, work * 16.0 * (double)n * (k + 3), work * 16.0 * c->V * 12 * (k + 1));
   auto vl = make_df_list(v, k);
   const dim3 g2(grid, B.n);
   const BatchDev bd = dev_of(B, n);
   switch (K) {
+    case 1: df_axpy_norm_dot_kernel<1><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
     case 4: df_axpy_norm_dot_kernel<4><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
     case 8: df_axpy_norm_dot_kernel<8><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;
     case 16: df_axpy_norm_dot_kernel<16><<<g2, kBlasThreads, 0, s>>>(vl, k, d_coef, w, rho, n, cond, part, d_out, bd); break;

@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(2 * kPairSites, QCD_PAIR_MIN_CTAS) dirac_pair_
 // clover as (hi, lo) pairs of FP32 values (the FP64 layouts with float4 =
 // (re hi, re lo, im hi, im lo) per complex number), computed on the FP32
 // units with error-free transformations.  Every output real is a double-float
-// running sum (dfacc); a hop's projection adds pairs by TwoSum, its SU(3)
+// running sum; a hop's projection adds pairs by TwoSum, its SU(3)
 // product accumulates exact FP32 products and their cross terms, its
 // expansion and the -1/2 (a power of two) are exact.  About 12 FP32 operations
 // per real multiply-add in place of one FP64 fused multiply-add, on units 64
@@ -369,45 +369,6 @@ __global__ void __launch_bounds__(2 * kPairSites, QCD_PAIR_MIN_CTAS) dirac_pair_
 // so are the results to the last rounding.  32^3 x 64 with an FP32 input: 1.41 ->
 // 1.09 ms, and 0.96 ms with the hops' data asked for ahead in registers (below);
 // on 8^3 x 16 34 -> 17 us.  The FMA pipe alone needs 0.69 ms.
-struct df2 {  // two double-floats
-  float2 hi, lo;
-};
-struct acc2 {  // two running sums (dfacc)
-  float2 s, c;
-};
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-// s + e = a + b exactly
-__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
-  s = add2(a, b);
-  const float2 bb = sub2(s, a);
-  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-}
-// a = x y, a += x y for double-floats x, y (x.lo y.lo dropped; YLO: y.lo is not 0)
-template <bool YLO>
-__device__ __forceinline__ void acc2_set(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
-  const float2 p = __fmul2_rn(xh, yh);
-  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
-  if (YLO) e = __ffma2_rn(xh, yl, e);
-  a = {p, e};
-}
-template <bool YLO>
-__device__ __forceinline__ void acc2_prod(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
-  const float2 p = __fmul2_rn(xh, yh);
-  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
-  if (YLO) e = __ffma2_rn(xh, yl, e);
-  float2 t;
-  two_sum2(a.s, p, a.s, t);
-  a.c = add2(a.c, add2(t, e));
-}
-// a += f z for f = +-1/2 (exact)
-__device__ __forceinline__ void acc2_add(acc2& a, float2 f, const acc2& z) {
-  float2 t;
-  two_sum2(a.s, __fmul2_rn(f, z.s), a.s, t);
-  a.c = add2(a.c, add2(t, __fmul2_rn(f, z.c)));
-}
-
 // the 24 output reals of a site: [spin pair][colour], lanes = the pair's spins
 struct SpinAcc {
   acc2 re[2][3], im[2][3];

@@ -110,28 +110,49 @@ __device__ __forceinline__ df df_fma(df x, df y, df z) {
   return fast_two_sum(s.hi, s.lo);
 }
 
-// A double-float running sum for long dot products: the high parts of the
-// terms are added by TwoSum, every lower-order term (a product's rounding
-// error, the cross terms, the sums' errors) is collected in c.  Neither part
-// is renormalised until the value is read.
-struct dfacc {
-  float s, c;
+// The same on packed FP32x2 instructions, two values at a time, with running
+// sums for long dot products: the high parts of the terms are added by TwoSum,
+// every lower-order term (a product's rounding error, the cross terms, the sums'
+// errors) is collected in c, and neither part is renormalised until it is read.
+__device__ __forceinline__ float2 bc2(float x) { return make_float2(x, x); }
+struct df2 {  // two double-floats
+  float2 hi, lo;
 };
-// a += x y for double-floats x = (xh, xl), y = (yh, yl) (xl yl dropped)
-__device__ __forceinline__ void acc_prod(dfacc& a, float xh, float xl, float yh, float yl) {
-  const df p = two_prod(xh, yh);
-  const df t = two_sum(a.s, p.hi);
-  a.s = t.hi;
-  a.c += t.lo + fmaf(xh, yl, fmaf(xl, yh, p.lo));
+struct acc2 {  // two running sums
+  float2 s, c;
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// s + e = a + b exactly
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = add2(a, b);
+  const float2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
-// a += (hi, lo)
-__device__ __forceinline__ void acc_add(dfacc& a, float hi, float lo) {
-  const df t = two_sum(a.s, hi);
-  a.s = t.hi;
-  a.c += t.lo + lo;
+// a = x y, a += x y for double-floats x, y (x.lo y.lo dropped; YLO: y.lo is not 0)
+template <bool YLO>
+__device__ __forceinline__ void acc2_set(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
+  const float2 p = __fmul2_rn(xh, yh);
+  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
+  if (YLO) e = __ffma2_rn(xh, yl, e);
+  a = {p, e};
 }
-__device__ __forceinline__ double acc_value(const dfacc& a) { return f32_to_f64(a.s) + f32_to_f64(a.c); }
-__device__ __forceinline__ df acc_df(const dfacc& a) { return two_sum(a.s, a.c); }
+template <bool YLO>
+__device__ __forceinline__ void acc2_prod(acc2& a, float2 xh, float2 xl, float2 yh, float2 yl) {
+  const float2 p = __fmul2_rn(xh, yh);
+  float2 e = __ffma2_rn(xl, yh, __ffma2_rn(xh, yh, neg2(p)));
+  if (YLO) e = __ffma2_rn(xh, yl, e);
+  float2 t;
+  two_sum2(a.s, p, a.s, t);
+  a.c = add2(a.c, add2(t, e));
+}
+// a += f z for f = +-1/2 (exact)
+__device__ __forceinline__ void acc2_add(acc2& a, float2 f, const acc2& z) {
+  float2 t;
+  two_sum2(a.s, __fmul2_rn(f, z.s), a.s, t);
+  a.c = add2(a.c, add2(t, __fmul2_rn(f, z.c)));
+}
 
 // ------------------------------------------------------------------------
 // complex arithmetic
@@ -240,7 +261,6 @@ __device__ __forceinline__ Half<T> udmul(const SU3<T>& u, const Half<T>& h) {
 // FP32 overloads on packed FP32x2 arithmetic (sm_100 family): the two spin
 // components of h travel in the two lanes, so each multiply-add by a link
 // entry (broadcast to both lanes) serves both components.
-__device__ __forceinline__ float2 bc2(float x) { return make_float2(x, x); }
 
 __device__ __forceinline__ Half<float> umul(const SU3<float>& u, const Half<float>& h) {
   float2 hr[3], hi[3];
