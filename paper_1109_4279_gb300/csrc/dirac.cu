@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(kDfThreads, 2) residual_df_kernel(Geom g, cons
 // r = b - D x (FP64), partial[blockIdx.x] = sum |r|^2 over the CTA; blockIdx.y
 // selects a right-hand side of a batch (fields V sites apart, partial sums ps
 // doubles apart), skipped when masked out
-__global__ void __launch_bounds__(256) residual64_kernel(Geom g, const void* __restrict__ U, FieldPtr A, FieldPtr b,
+__global__ void __launch_bounds__(kF64Threads) residual64_kernel(Geom g, const void* __restrict__ U, FieldPtr A, FieldPtr b,
                                                          FieldPtr x, FieldPtr r_out, double* partial, long long ps,
                                                          const int* __restrict__ mask) {
   __shared__ double sh[32];
@@ -881,11 +881,11 @@ int residual64(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec& 
   if (b.prec != P64 || x.prec != P64 || r.prec != P64) return QCD_ERR_ARG;
   QCD_TRY(ensure_gauge(c, P64, s));
   QCD_TRY(ensure_clover(c, P64, s));
-  const unsigned grid = (unsigned)((c->V + 255) / 256);
+  const unsigned grid = (unsigned)((c->V + kF64Threads - 1) / kF64Threads);
   {
     ProfScope ps(c, QCD_KERNEL_RESIDUAL, s, (bytes_per_site(P64) + 192) * (double)c->V * B.n,
                  1848.0 * (double)c->V * B.n);
-    residual64_kernel<<<dim3(grid, B.n), 256, 0, s>>>(c->g, c->U[P64], c->A[P64].ptr(), b.ptr(), x.ptr(), r.ptr(),
+    residual64_kernel<<<dim3(grid, B.n), kF64Threads, 0, s>>>(c->g, c->U[P64], c->A[P64].ptr(), b.ptr(), x.ptr(), r.ptr(),
                                                        part + kPartHead, B.ps, B.mask);
     QCD_LAUNCHED();
   }
@@ -924,7 +924,7 @@ int residual_df(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec&
 // the load of x.  FP64 throughout.
 // ------------------------------------------------------------------------
 template <int DAG, int PRE, int USE_M>
-__global__ void __launch_bounds__(256, 2) eo_kernel(Geom g, const void* __restrict__ U, FieldPtr Ahat, FieldPtr x,
+__global__ void __launch_bounds__(kF64Threads, 8) eo_kernel(Geom g, const void* __restrict__ U, FieldPtr Ahat, FieldPtr x,
                                                  FieldPtr y, FieldPtr out, int par, double c1, double c2) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.V / 2) return;
@@ -962,7 +962,7 @@ int eo_apply(qcd_ctx* c, const Rec& x, const Rec& y, const Rec& out, int par, in
   if (x.prec != P64 || y.prec != P64 || out.prec != P64 || (par != 0 && par != 1)) return QCD_ERR_ARG;
   QCD_TRY(ensure_gauge(c, P64, s));
   QCD_TRY(ensure_clover(c, P64, s));
-  const unsigned grid = (unsigned)((c->V / 2 + 255) / 256);
+  const unsigned grid = (unsigned)((c->V / 2 + kF64Threads - 1) / kF64Threads);
   // algorithmic bytes: per site of parity par, 8 neighbour spinors and 8 links
   // (hops), x and the clover record (if used) and the result
   const double sites = (double)c->V / 2;
@@ -970,7 +970,7 @@ int eo_apply(qcd_ctx* c, const Rec& x, const Rec& y, const Rec& out, int par, in
   ProfScope ps(c, QCD_KERNEL_DIRAC, s, bytes, sites * ((c2 != 0.0 ? 1320.0 : 0.0) + (use_m ? 504.0 : 0.0)));
   const void* U = c->U[P64];
   const FieldPtr A = c->Ahat[P64].ptr();
-#define EO(D, P, M) eo_kernel<D, P, M><<<grid, 256, 0, s>>>(c->g, U, A, x.ptr(), y.ptr(), out.ptr(), par, c1, c2)
+#define EO(D, P, M) eo_kernel<D, P, M><<<grid, kF64Threads, 0, s>>>(c->g, U, A, x.ptr(), y.ptr(), out.ptr(), par, c1, c2)
   if (dagger) {
     if (pre) { if (use_m) EO(1, 1, 1); else EO(1, 1, 0); }
     else { if (use_m) EO(1, 0, 1); else EO(1, 0, 0); }

@@ -44,6 +44,9 @@ inline int chunks(int prec, int nreal) {
 // CTA size of the double-float kernels: their registers allow 8 warps per SM, and
 // two CTAs of four fill an SM's gaps better than one of eight
 static constexpr int kDfThreads = 128;
+// and of the FP64 ones: a warp's operation holds a quarter of an SM's FP64 unit for
+// 64 cycles, so a small lattice's warps have to be spread over the quarters
+static constexpr int kF64Threads = 64;
 
 // doubles at the start of every right-hand side's partial sums; the first word is
 // the count of finished CTAs, 0 between kernels
@@ -183,7 +186,10 @@ struct qcd_ctx {
   qcd::Timer timers[QCD_KERNEL_COUNT];
   std::vector<cudaEvent_t> event_pool;
   // launch shape chosen by the autotuner
-  int dirac_threads[5] = {256, 256, 256, 256, qcd::kDfThreads};  // CTA size of the operator kernel per precision
+  // CTA size of the operator kernel per precision.  Small CTAs spread a small lattice
+  // over the SMs and leave a smaller last wave (FP64 on 16^3 x 32 271 us with 64
+  // threads, 305 with 256, on 8^4 43 and 79; 16-bit storage 15.2 and 16.9).
+  int dirac_threads[5] = {64, 128, 128, 128, qcd::kDfThreads};
   int sap_rt = 0;  // right-hand sides per CTA of batched SAP launches (0: sap_tile's default)
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)
   double* d_scalars = nullptr;  // small device array for coefficients
