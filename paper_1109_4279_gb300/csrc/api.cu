@@ -34,6 +34,44 @@ int rec_alloc(Rec& r, int prec, int nreal, long long V) {
   return QCD_OK;
 }
 
+size_t rec_bytes(int prec, int nreal, long long V) {
+  return (size_t)V * chunks(prec, nreal) * 16 + ((prec == P16 || prec == PB16) ? (size_t)V * sizeof(float) : 0);
+}
+
+Rec rec_view(void* p, int prec, int nreal, long long V) {
+  Rec r;
+  const size_t data = (size_t)V * chunks(prec, nreal) * 16;
+  r.prec = prec;
+  r.nreal = nreal;
+  r.data = p;
+  r.norm = (prec == P16 || prec == PB16) ? (float*)((char*)p + data) : nullptr;
+  r.bytes = rec_bytes(prec, nreal, V);
+  return r;
+}
+
+int Scratch::get(qcd_ctx* c, int slot, size_t bytes) {
+  if (bytes <= c->scratch_bytes[slot]) {
+    p = c->scratch[slot];
+    return QCD_OK;
+  }
+  own = bytes > kScratchKeep;
+  if (!own) {  // replaces the slot's smaller buffer (no call is using it)
+    if (c->scratch[slot]) cudaFree(c->scratch[slot]);
+    c->scratch[slot] = nullptr;
+    c->scratch_bytes[slot] = 0;
+  }
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+    return QCD_ERR_NOMEM;
+  }
+  if (!own) {
+    c->scratch[slot] = p;
+    c->scratch_bytes[slot] = bytes;
+  }
+  return QCD_OK;
+}
+
 void rec_free(Rec& r) {
   if (r.data) cudaFree(r.data);
   r = Rec();
@@ -176,6 +214,8 @@ void qcd_destroy(qcd_ctx* c) {
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
   if (c->deliver_stream) cudaStreamDestroy(c->deliver_stream);
   c->streams.clear();
+  for (void* p : c->scratch)
+    if (p) cudaFree(p);
   if (c->d_tables) cudaFree(c->d_tables);
   if (c->d_scalars) cudaFree(c->d_scalars);
   if (c->h_scalars) cudaFreeHost(c->h_scalars);
@@ -216,15 +256,14 @@ int qcd_apply_D(qcd_ctx* c, const double* in, double* out, int dagger, int prec,
   if (!c || !in || !out || nrhs < 1 || prec < 0 || prec > 4) return QCD_ERR_ARG;
   if (!c->clover_built) return QCD_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
-  Rec a, b;
-  int st = rec_alloc(a, prec, 24, c->V * nrhs);
-  if (st == QCD_OK) st = rec_alloc(b, prec, 24, c->V * nrhs);
-  if (st == QCD_OK) st = import_spinor(c, in, a, nrhs, s);
+  const size_t bytes = (rec_bytes(prec, 24, c->V * nrhs) + 255) / 256 * 256;
+  Scratch mem;
+  QCD_TRY(mem.get(c, kScratchFields, 2 * bytes));
+  const Rec a = rec_view(mem.p, prec, 24, c->V * nrhs), b = rec_view((char*)mem.p + bytes, prec, 24, c->V * nrhs);
+  int st = import_spinor(c, in, a, nrhs, s);
   if (st == QCD_OK) st = dirac_apply(c, a, b, dagger, s, nrhs);
   if (st == QCD_OK) st = export_spinor(c, b, out, nrhs, s);
   cudaStreamSynchronize(s);
-  rec_free(a);
-  rec_free(b);
   return st;
 }
 
@@ -549,15 +588,14 @@ int qcd_force(qcd_ctx* c, const double* x, const double* y, double* F, void* str
   if (!c || !x || !y || !F) return QCD_ERR_ARG;
   if (!c->clover_built) return QCD_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
-  Rec xi, yi;
-  int st = rec_alloc(xi, P64, 24, c->V);
-  if (st == QCD_OK) st = rec_alloc(yi, P64, 24, c->V);
-  if (st == QCD_OK) st = import_spinor(c, x, xi, 1, s);
+  const size_t bytes = rec_bytes(P64, 24, c->V);  // (a multiple of 256: V is one of 16)
+  Scratch mem;
+  QCD_TRY(mem.get(c, kScratchFields, 2 * bytes));
+  const Rec xi = rec_view(mem.p, P64, 24, c->V), yi = rec_view((char*)mem.p + bytes, P64, 24, c->V);
+  int st = import_spinor(c, x, xi, 1, s);
   if (st == QCD_OK) st = import_spinor(c, y, yi, 1, s);
   if (st == QCD_OK) st = force_apply(c, xi, yi, F, s);
   cudaStreamSynchronize(s);
-  rec_free(xi);
-  rec_free(yi);
   return st;
 }
 
@@ -574,9 +612,10 @@ int qcd_gradient(qcd_ctx* c, const double* phi, double* dL_dphi, double* dL_dthe
   for (Rec* f : {&w->b, &w->x})
     if (!f->data) QCD_TRY(rec_alloc(*f, P64, 24, c->V));
   const size_t fbytes = (size_t)c->V * 24 * sizeof(double);
-  Rec xk, yk;
-  int st = rec_alloc(xk, P64, 24, c->V);
-  if (st == QCD_OK) st = rec_alloc(yk, P64, 24, c->V);
+  Scratch mem;
+  QCD_TRY(mem.get(c, kScratchFields, 2 * fbytes));
+  const Rec xk = rec_view(mem.p, P64, 24, c->V), yk = rec_view((char*)mem.p + fbytes, P64, 24, c->V);
+  int st = QCD_OK;
   // x = D^-1 phi
   if (st == QCD_OK) st = import_spinor(c, phi, w->b, 1, s);
   if (st == QCD_OK) st = cudaMemsetAsync(xk.data, 0, fbytes, s) == cudaSuccess ? QCD_OK : QCD_ERR_CUDA;
@@ -599,8 +638,6 @@ int qcd_gradient(qcd_ctx* c, const double* phi, double* dL_dphi, double* dL_dthe
     if (st == QCD_OK) st = export_spinor(c, xk, dL_dphi, 1, s);
   }
   cudaStreamSynchronize(s);
-  rec_free(xk);
-  rec_free(yk);
   return st;
 }
 

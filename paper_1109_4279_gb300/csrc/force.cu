@@ -412,11 +412,9 @@ int force_apply(qcd_ctx* c, const Rec& x, const Rec& y, double* F, cudaStream_t 
   const size_t per_plane = (size_t)c->V * 41 * sizeof(double);
   const int group = 6 * per_plane <= ((size_t)4 << 30) ? 6 : 1;
   const bool clover = c->p.csw != 0.0;
-  double* W = nullptr;
-  if (clover && cudaMalloc(&W, per_plane * group) != cudaSuccess) {
-    cudaGetLastError();
-    return QCD_ERR_NOMEM;
-  }
+  Scratch mem;
+  if (clover) QCD_TRY(mem.get(c, kScratchForce, per_plane * group));
+  double* W = (double*)mem.p;
   double* S = W + (size_t)c->V * 9 * group;
   const unsigned grid = (unsigned)((c->V + 127) / 128);
   const double2* U = (const double2*)c->U[P64];
@@ -442,7 +440,6 @@ int force_apply(qcd_ctx* c, const Rec& x, const Rec& y, double* F, cudaStream_t 
     if (!clover) break;
   }
   cudaStreamSynchronize(s);
-  if (W) cudaFree(W);
   return st;
 }
 

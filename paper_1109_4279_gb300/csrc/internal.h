@@ -192,6 +192,8 @@ struct qcd_ctx {
   int dirac_threads[5] = {64, 128, 128, 128, qcd::kDfThreads};
   int sap_rt = 0;  // right-hand sides per CTA of batched SAP launches (0: sap_tile's default)
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)
+  void* scratch[2] = {nullptr, nullptr};  // kept staging buffers (qcd::Scratch)
+  size_t scratch_bytes[2] = {0, 0};
   double* d_scalars = nullptr;  // small device array for coefficients
   double* h_scalars = nullptr;  // pinned host mirror
   // test hooks (qcd_debug_set): budget of the SAP staging wait, and bytes its
@@ -228,6 +230,28 @@ struct ProfScope {
 };
 
 // ---- memory helpers (api.cu)
+// Staging memory of a context for entry points that need fields or scratch only
+// while they run (cudaMalloc and cudaFree took 100 to 300 us of each such call).
+// A slot's buffer is kept for the next call -- every such entry point waits for
+// its work before it returns, so calls on different streams do not share it at
+// the same time -- up to kScratchKeep bytes; larger requests are allocated and
+// freed by the call as before.  Freed with the context.
+static constexpr size_t kScratchKeep = (size_t)1 << 30;
+struct Scratch {
+  void* p = nullptr;
+  bool own = false;  // allocated for this call alone
+  Scratch() = default;
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  ~Scratch() {
+    if (own && p) cudaFree(p);
+  }
+  int get(qcd_ctx* c, int slot, size_t bytes);
+};
+enum { kScratchFields = 0, kScratchForce = 1, kScratchSlots = 2 };
+// bytes of a record field, and a view of one on memory that rec_free must not see
+size_t rec_bytes(int prec, int nreal, long long V);
+Rec rec_view(void* p, int prec, int nreal, long long V);
 int rec_alloc(Rec& r, int prec, int nreal, long long V);
 void rec_free(Rec& r);
 Workspace* ensure_ws(qcd_ctx* c);
