@@ -775,6 +775,134 @@ __global__ void __launch_bounds__(kF64Threads) residual64_kernel(Geom g, const v
   if (threadIdx.x == 0) partial[blockIdx.x] = t;
 }
 
+// ------------------------------------------------------------------------
+// The FP64 operator with a site's work split over the four warps of a CTA of 32
+// sites, for lattices whose sites alone do not keep the FP64 units busy: a warp's
+// FP64 operation holds a quarter of an SM for 64 cycles, so one thread's 1150 of
+// them last 36 us however few warps there are.  Warp w computes the two hops of
+// direction w; the partial sums meet in shared memory, and warp w finishes spin w
+// (its three rows of the chiral clover block).  RES: out = b - D x and the sum of
+// its squares per CTA instead of out = D x.
+// ------------------------------------------------------------------------
+static constexpr int kSplitSites = 32;
+
+// rows R0 .. R0 + 2 of a packed Hermitian 6x6 block (chunks of record a) times in
+template <int R0>
+__device__ __forceinline__ void clover_rows(const double2* __restrict__ a, int Vb, const cpx<double>* in,
+                                            cpx<double>* out) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int i = R0 + c;
+    const double2 dv = __ldg(a + (long long)(i >> 1) * Vb);
+    out[c] = ((i & 1) ? dv.y : dv.x) * in[i];
+  }
+  int k = 3;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i + 1; j < 6; ++j, ++k) {
+      const bool row_i = i >= R0 && i < R0 + 3, row_j = j >= R0 && j < R0 + 3;
+      if (!row_i && !row_j) continue;
+      const double2 v = __ldg(a + (long long)k * Vb);
+      const cpx<double> e = {v.x, v.y};
+      if (row_i) out[i - R0] = cmadd(e, in[j], out[i - R0]);
+      if (row_j) out[j - R0] = cjmadd(e, in[i], out[j - R0]);
+    }
+}
+
+template <int DAG, bool RES>
+__global__ void __launch_bounds__(4 * kSplitSites, 4) dirac_split_kernel(Geom g, const void* __restrict__ U, FieldPtr A,
+                                                                         FieldPtr in, FieldPtr out, FieldPtr b,
+                                                                         const int* __restrict__ mask, int out_df,
+                                                                         double* partial, long long ps) {
+  __shared__ double part[4][24][kSplitSites];
+  __shared__ double sh[4];
+  if (mask && !mask[blockIdx.y]) return;
+  const long long fo = (long long)blockIdx.y * g.V * 12;  // 16-byte chunks per field
+  in.data = (double2*)in.data + fo;
+  out.data = (double2*)out.data + fo;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const long long s0 = (long long)blockIdx.x * kSplitSites + l;
+  const bool on = s0 < g.V;
+  const long long s = on ? s0 : 0;
+  const int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
+  {
+    int n[4], y[4];
+    block_coords(g, blk, n);
+    const int packed = __ldg(g.r2y + r);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) y[mu] = ycoord(packed, mu);
+    Spinor<double> acc;
+    zero(acc);
+    switch (w) {
+      case 0: hop_pair<0, P64, DAG, double>(g, U, in, blk, r, y, n, acc); break;
+      case 1: hop_pair<1, P64, DAG, double>(g, U, in, blk, r, y, n, acc); break;
+      case 2: hop_pair<2, P64, DAG, double>(g, U, in, blk, r, y, n, acc); break;
+      default: hop_pair<3, P64, DAG, double>(g, U, in, blk, r, y, n, acc); break;
+    }
+#pragma unroll
+    for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        part[w][6 * sp + 2 * c][l] = acc.c[sp][c].re;
+        part[w][6 * sp + 2 * c + 1][l] = acc.c[sp][c].im;
+      }
+  }
+  // spin w: its clover rows while the other warps arrive
+  const int hb = w >> 1;
+  cpx<double> psi[6], o[3];
+  const double2* f = (const double2*)in.data + ((long long)blk * 12 + 6 * hb) * g.Vb + r;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const double2 v = __ldg(f + (long long)k * g.Vb);
+    psi[k] = {v.x, v.y};
+  }
+  const double2* a = (const double2*)A.data + ((long long)blk * 36 + 18 * hb) * g.Vb + r;
+  if (w & 1)
+    clover_rows<3>(a, g.Vb, psi, o);
+  else
+    clover_rows<0>(a, g.Vb, psi, o);
+  __syncthreads();
+  double nrm = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int e = 6 * w + 2 * c;
+    cpx<double> h = {part[0][e][l], part[0][e + 1][l]};
+#pragma unroll
+    for (int q = 1; q < 4; ++q) h = h + cpx<double>{part[q][e][l], part[q][e + 1][l]};
+    h = h + o[c];
+    const long long at = ((long long)blk * 12 + 3 * w + c) * g.Vb + r;
+    if (RES) {
+      const double2 bv = __ldg((const double2*)b.data + fo + at);
+      h = cpx<double>{bv.x, bv.y} - h;
+      if (on) nrm += h.re * h.re + h.im * h.im;
+    }
+    if (!on) continue;
+    if (out_df) {
+      const df x = df_from_f64(h.re), y = df_from_f64(h.im);
+      ((float4*)out.data)[at] = make_float4(x.hi, x.lo, y.hi, y.lo);
+    } else {
+      ((double2*)out.data)[at] = make_double2(h.re, h.im);
+    }
+  }
+  if (RES) {
+    const double t = block_sum(nrm, sh);
+    if (threadIdx.x == 0) partial[blockIdx.y * ps + blockIdx.x] = t;
+  }
+}
+
+// The split form where its warps fill the SM quarters better: FP64 operations that
+// one quarter runs through, per warp 1150 (one thread per site, right-hand sides in
+// turn) or 306 (split, right-hand sides side by side), times the warps it gets.
+// One right-hand side, one thread per site / split: 256 sites 41 / 15 us, 8192 43 / 25,
+// 16384 43 / 45, 32768 80 / 74, 41472 107 / 94, 65536 147 / 146, 131072 271 / 275.
+static bool use_split(const qcd_ctx* c, int nrhs) {
+  if (nrhs > 65535) return false;  // (a grid dimension)
+  const long long q = 4LL * c->sms;
+  const long long whole = (c->V + 32 * q - 1) / (32 * q) * nrhs, split = (c->V * nrhs + 8 * q - 1) / (8 * q);
+  return split * 306 < whole * 1150;
+}
+
 static double bytes_per_site(int prec) {
   if (prec == P64) return 2 * 24 * 8 + 4 * 18 * 8 + 72 * 8;
   if (prec == P32) return 2 * 24 * 4 + 4 * 12 * 4 + 72 * 4;
@@ -847,6 +975,17 @@ int dirac_apply(qcd_ctx* c, const Rec& in, const Rec& out, int dagger, cudaStrea
     QCD_LAUNCHED();
     return QCD_OK;
   }
+  if (prec == P64 && use_split(c, nrhs)) {
+    const dim3 g2((unsigned)((c->V + kSplitSites - 1) / kSplitSites), nrhs);
+    if (dagger)
+      dirac_split_kernel<1, false><<<g2, 4 * kSplitSites, 0, s>>>(c->g, U, A, in.ptr(), out.ptr(), FieldPtr{}, mask,
+                                                                  out_df, nullptr, 0);
+    else
+      dirac_split_kernel<0, false><<<g2, 4 * kSplitSites, 0, s>>>(c->g, U, A, in.ptr(), out.ptr(), FieldPtr{}, mask,
+                                                                  out_df, nullptr, 0);
+    QCD_LAUNCHED();
+    return QCD_OK;
+  }
   switch (prec) {
     case P64: LAUNCH(P64, 0); break;
     case P32: LAUNCH(P32, 0); break;
@@ -881,11 +1020,17 @@ int residual64(qcd_ctx* c, double* part, const Rec& b, const Rec& x, const Rec& 
   if (b.prec != P64 || x.prec != P64 || r.prec != P64) return QCD_ERR_ARG;
   QCD_TRY(ensure_gauge(c, P64, s));
   QCD_TRY(ensure_clover(c, P64, s));
-  const unsigned grid = (unsigned)((c->V + kF64Threads - 1) / kF64Threads);
+  const bool split = use_split(c, B.n);
+  const int sites = split ? kSplitSites : kF64Threads;  // per CTA
+  const unsigned grid = (unsigned)((c->V + sites - 1) / sites);
   {
     ProfScope ps(c, QCD_KERNEL_RESIDUAL, s, (bytes_per_site(P64) + 192) * (double)c->V * B.n,
                  1848.0 * (double)c->V * B.n);
-    residual64_kernel<<<dim3(grid, B.n), kF64Threads, 0, s>>>(c->g, c->U[P64], c->A[P64].ptr(), b.ptr(), x.ptr(), r.ptr(),
+    if (split)
+      dirac_split_kernel<0, true><<<dim3(grid, B.n), 4 * kSplitSites, 0, s>>>(
+          c->g, c->U[P64], c->A[P64].ptr(), x.ptr(), r.ptr(), b.ptr(), B.mask, 0, part + kPartHead, B.ps);
+    else
+      residual64_kernel<<<dim3(grid, B.n), kF64Threads, 0, s>>>(c->g, c->U[P64], c->A[P64].ptr(), b.ptr(), x.ptr(), r.ptr(),
                                                        part + kPartHead, B.ps, B.mask);
     QCD_LAUNCHED();
   }

@@ -42,7 +42,7 @@ namespace qcd {
 
 size_t partials_for(long long V) {
   const size_t blas = (size_t)152 * 8 * 65;     // largest BLAS grid x widest record
-  const size_t resid = (size_t)(V + kF64Threads - 1) / kF64Threads;  // one partial per residual CTA
+  const size_t resid = (size_t)(V + 31) / 32;  // one partial per residual CTA (of 32 sites at least)
   return kPartHead + (blas > resid ? blas : resid);
 }
 
