@@ -49,27 +49,49 @@ Rec rec_view(void* p, int prec, int nreal, long long V) {
   return r;
 }
 
-int Scratch::get(qcd_ctx* c, int slot, size_t bytes) {
-  if (bytes <= c->scratch_bytes[slot]) {
-    p = c->scratch[slot];
-    return QCD_OK;
-  }
-  own = bytes > kScratchKeep;
-  if (!own) {  // replaces the slot's smaller buffer (no call is using it)
+// frees the kept buffer of a slot that no call holds
+static void scratch_drop(qcd_ctx* c, int slot) {
+  if (c->scratch_busy[slot].exchange(1)) return;
+  if (c->scratch[slot]) cudaFree(c->scratch[slot]);
+  c->scratch[slot] = nullptr;
+  c->scratch_bytes[slot] = 0;
+  c->scratch_busy[slot].store(0);
+}
+
+int Scratch::get(qcd_ctx* c, int slot_, size_t bytes) {
+  slot = slot_;
+  if (bytes <= kScratchKeep && !c->scratch_busy[slot].exchange(1)) {
+    claimed = c;
+    if (bytes <= c->scratch_bytes[slot]) {
+      p = c->scratch[slot];
+      return QCD_OK;
+    }
     if (c->scratch[slot]) cudaFree(c->scratch[slot]);
     c->scratch[slot] = nullptr;
     c->scratch_bytes[slot] = 0;
   }
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {  // once more without what the context keeps
+    cudaGetLastError();
+    for (int k = 0; k < kScratchSlots; ++k) scratch_drop(c, k);
+    e = cudaMalloc(&p, bytes);
+  }
+  if (e != cudaSuccess) {
     cudaGetLastError();
     p = nullptr;
     return QCD_ERR_NOMEM;
   }
-  if (!own) {
+  own = !claimed;
+  if (claimed) {
     c->scratch[slot] = p;
     c->scratch_bytes[slot] = bytes;
   }
   return QCD_OK;
+}
+
+Scratch::~Scratch() {
+  if (own) cudaFree(p);
+  if (claimed) claimed->scratch_busy[slot].store(0);
 }
 
 void rec_free(Rec& r) {

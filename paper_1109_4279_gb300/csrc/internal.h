@@ -194,6 +194,7 @@ struct qcd_ctx {
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)
   void* scratch[2] = {nullptr, nullptr};  // kept staging buffers (qcd::Scratch)
   size_t scratch_bytes[2] = {0, 0};
+  std::atomic<int> scratch_busy[2] = {{0}, {0}};  // a call holds the slot
   double* d_scalars = nullptr;  // small device array for coefficients
   double* h_scalars = nullptr;  // pinned host mirror
   // test hooks (qcd_debug_set): budget of the SAP staging wait, and bytes its
@@ -232,20 +233,21 @@ struct ProfScope {
 // ---- memory helpers (api.cu)
 // Staging memory of a context for entry points that need fields or scratch only
 // while they run (cudaMalloc and cudaFree took 100 to 300 us of each such call).
-// A slot's buffer is kept for the next call -- every such entry point waits for
-// its work before it returns, so calls on different streams do not share it at
-// the same time -- up to kScratchKeep bytes; larger requests are allocated and
-// freed by the call as before.  Freed with the context.
+// A slot's buffer of up to kScratchKeep bytes is kept for the next call.  A call
+// claims the slot until it returns, and every such entry point waits for its work
+// before that, so calls on different streams never share the buffer; a call that
+// finds the slot claimed (another thread's) and one that wants more allocates and
+// frees its own.  Freed with the context, or when an allocation here fails.
 static constexpr size_t kScratchKeep = (size_t)1 << 30;
 struct Scratch {
   void* p = nullptr;
-  bool own = false;  // allocated for this call alone
+  bool own = false;           // allocated for this call alone
+  qcd_ctx* claimed = nullptr;  // the context whose slot this call holds
+  int slot = 0;
   Scratch() = default;
   Scratch(const Scratch&) = delete;
   Scratch& operator=(const Scratch&) = delete;
-  ~Scratch() {
-    if (own && p) cudaFree(p);
-  }
+  ~Scratch();
   int get(qcd_ctx* c, int slot, size_t bytes);
 };
 enum { kScratchFields = 0, kScratchForce = 1, kScratchSlots = 2 };

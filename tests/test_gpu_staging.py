@@ -1,7 +1,10 @@
 """Entry points that stage fields in memory kept by the context: calls of
-changing size and precision one after another, on two streams, and one whose
-fields exceed what is kept, give what a fresh context gives.
+changing size and precision one after another, on two streams, one whose
+fields exceed what is kept, and calls from several threads at the same time,
+give what a fresh context gives.
 """
+import threading
+
 import pytest
 
 from paper_1109_4279_gb300 import synth
@@ -59,4 +62,37 @@ def test_fields_beyond_what_is_kept():
         one = torch.empty_like(psi[0])
         binding.qcd_apply_D(lat.ctx, psi[k].contiguous(), one)
         assert torch.equal(one, out[k])
+    lat.close()
+
+
+def test_threads_do_not_share_the_memory():
+    """Four threads apply D of one context on their own streams at the same time;
+    each gets its own answer (the kernels sum in a fixed order: bit for bit)."""
+    from paper_1109_4279_gb300 import binding
+    dims, block, n = (16, 8, 8, 8), (4, 4, 4, 4), 4
+    U, rng = synth.gauge_field(dims, 0.5, 32)
+    lat = _lattice(dims, block, torch.from_numpy(U).cuda())
+    psi = torch.from_numpy(synth.gaussian_spinor(dims, rng, nrhs=n)).cuda()
+    want = [lat.apply_D(psi[k], prec="f64") for k in range(n)]
+    outs = [[torch.empty_like(psi[k]) for _ in range(12)] for k in range(n)]
+    streams = [torch.cuda.Stream() for _ in range(n)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            with torch.cuda.stream(streams[k]):
+                for o in outs[k]:
+                    binding.qcd_apply_D(lat.ctx, psi[k], o)
+        except Exception as e:  # (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(n)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    assert all(torch.equal(o, want[k]) for k in range(n) for o in outs[k])
     lat.close()
