@@ -28,6 +28,8 @@
  *             rows and rebuild the third);
  *   force     (V, 4 mu, 8) float64: dL/dtheta_a for U_mu(x) ->
  *             exp(i theta_a lambda_a / 2) U_mu(x), Gell-Mann lambda_a.
+ * Arrays of complex numbers start on a 16-byte boundary (as torch and C align the
+ * type); real FP64 arrays (forces, momenta) on an 8-byte one.
  * Gamma matrices: chiral basis, g5 = g0 g1 g2 g3 = diag(1, 1, -1, -1),
  * g0 = [[0, -1], [-1, 0]], g_k = [[0, -i s_k], [i s_k, 0]] (2x2 blocks).
  *

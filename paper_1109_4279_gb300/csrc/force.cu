@@ -348,7 +348,8 @@ __global__ void __launch_bounds__(128) force_kernel(Geom g, const double2* __res
   const int blk = (int)(s / g.Vb), r = (int)(s - (long long)blk * g.Vb);
   int x[4];
   global_coords(g, blk, r, x);
-  double2* o = (double2*)(F + (lex_index(g, x) * 4 + mu) * 8);
+  // F is a caller's array, aligned to 8 bytes only: one double at a time
+  double* o = F + (lex_index(g, x) * 4 + mu) * 8;
   double out[8];
   if (first) {
     const long long sp = shifted(g, x, mu, 1, -1, 0);
@@ -380,11 +381,7 @@ __global__ void __launch_bounds__(128) force_kernel(Geom g, const double2* __res
     for (int a = 0; a < 8; ++a) out[a] *= -0.25 * eta;
   } else {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double2 v = o[k];
-      out[2 * k] = v.x;
-      out[2 * k + 1] = v.y;
-    }
+    for (int k = 0; k < 8; ++k) out[k] = o[k];
   }
 #pragma unroll 1
   for (int q = 0; q < np; ++q) {
@@ -399,7 +396,7 @@ __global__ void __launch_bounds__(128) force_kernel(Geom g, const double2* __res
     for (int k = 0; k < 8; ++k) out[k] += __ldg(a + (long long)k * g.V) + __ldg(b + (long long)k * g.V);
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) o[k] = make_double2(out[2 * k], out[2 * k + 1]);
+  for (int k = 0; k < 8; ++k) o[k] = out[k];
 }
 
 int force_apply(qcd_ctx* c, const Rec& x, const Rec& y, double* F, cudaStream_t s) {

@@ -153,17 +153,13 @@ __global__ void __launch_bounds__(128) gauge_force_kernel(Lex g, const double2* 
   for (int a = 0; a < 8; ++a) F[l * 8 + a] = o[a];
 }
 
-// F of link l (+)= sg o
+// F of link l (+)= sg o; one double at a time (F is a caller's array, aligned to 8
+// bytes only)
 template <int FIRST>
 __device__ __forceinline__ void force_add(double* F, long long l, double sg, const double o[8]) {
-  double2* f = (double2*)(F + l * 8);
+  double* f = F + l * 8;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    double2 v = FIRST ? make_double2(0.0, 0.0) : f[k];
-    v.x += sg * o[2 * k];
-    v.y += sg * o[2 * k + 1];
-    f[k] = v;
-  }
+  for (int k = 0; k < 8; ++k) f[k] = (FIRST ? 0.0 : f[k]) + sg * o[k];
 }
 
 // The same force, one thread per plaquette (x; mu < nu).  Read from its corners
@@ -241,13 +237,9 @@ __global__ void __launch_bounds__(kThreads) link_update_kernel(long long nlinks,
                                                                const double* __restrict__ pi, double eps) {
   const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= nlinks) return;
-  double p[8];
+  double p[8];  // (pi, a caller's array, is aligned to 8 bytes only)
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const double2 v = ((const double2*)(pi + l * 8))[k];
-    p[2 * k] = v.x;
-    p[2 * k + 1] = v.y;
-  }
+  for (int k = 0; k < 8; ++k) p[k] = pi[l * 8 + k];
   const double r3 = 0.5773502691896257645;
   double h = 0.5 * eps;
   // H00 = h (p3 + p8/sqrt3), H11 = h (-p3 + p8/sqrt3), H22 = -2 h p8/sqrt3,
