@@ -1160,7 +1160,7 @@ __global__ void __launch_bounds__(SapThreads<P>::most) sap_sweep_kernel(SapArgs 
       rho_o = half_axpy(rho_o, half_axpy(half_of(po, hf), s_half(s_t, ns, re, hf), T(1)), T(1));
     }
     // etahat = rho_e - D_eo A_oo^-1 rho_o: first t = A_oo^-1 rho_o, which is also
-    // where chi_o starts
+    // where the sum for chi_o starts
     Half<T> chi_o = clover_half(st, ro, hf, rho_o);
     if (act) s_half_store(s_t, ns, i, hf, chi_o);
     __syncthreads();
@@ -1170,7 +1170,8 @@ __global__ void __launch_bounds__(SapThreads<P>::most) sap_sweep_kernel(SapArgs 
     for (int s = 0; s < 2; ++s)
 #pragma unroll
       for (int c = 0; c < 3; ++c) x.c[s][c] = {T(0), T(0)};
-    if (act) s_half_store(s_r, ns, i, hf, r);
+    constexpr bool kLinear = kHalf;  // (the MR steps below)
+    if (act) s_half_store(s_r, ns, i, hf, kLinear || a.nmr > 0 ? r : x);
     __syncthreads();
 
     if constexpr (kHalf) {
@@ -1179,71 +1180,117 @@ __global__ void __launch_bounds__(SapThreads<P>::most) sap_sweep_kernel(SapArgs 
 
     // ---- MR on Dhat = A_ee - D_eo A_oo^-1 D_oe from x_e = 0, r = etahat:
     //   t = A_oo^-1 D_oe r;  p = A_ee r - D_eo t;  a = (p, r) / |p|^2;
-    //   x += a r;  r -= a p.
-    // Two things follow from linearity.  t is updated with r, t -= a A_oo^-1 D_oe p,
-    // so p itself goes to shared memory and the next hops start before a is known:
-    // a step needs two CTA-wide barriers and no wait for the sums (three and one
-    // before).  And A_oo^-1 D_oe x = sum a t, so the back substitution chi_o = A_oo^-1 (rho_o - D_oe x_e) is one
-    // multiply-add per step instead of one more pass of hops.  Each step runs two
-    // phases through one code path: phase 0 (odd sites) t, phase 1 (even sites) p.
-    // With the loads ahead and the L2 prefetch, a launch on 32^3 x 64 in 8x4x4x4
-    // blocks went from 0.551 to 0.497 ms, for 12 right-hand sides on 24^3 x 48 from
-    // 2.30 to 1.95 ms.
-    cpx<T> alpha = {T(0), T(0)};
-    auto advance = [&] {  // with a of the finished step: x, r, chi_o (s_r holds p, s_t holds t)
-      T pr_re, pr_im, pp;
-      sum3_get(pr_re, pr_im, pp, s_red);
-      const T inv = pp > T(0) ? T(1) / pp : T(0);
-      alpha = {pr_re * inv, pr_im * inv};
-      const Half<T> p = s_half(s_r, ns, re, hf), t = s_half(s_t, ns, re, hf);
+    //   x += a r;  r -= a p;  at the end chi_o = A_oo^-1 (rho_o - D_oe x_e).
+    // Each step runs two phases through one code path: phase 0 (odd sites) t, phase
+    // 1 (even sites) p.
+    if constexpr (kLinear) {
+      // t is updated with r, t -= a A_oo^-1 D_oe p, so p itself goes to shared memory
+      // and the next hops start before a is known: a step needs two CTA-wide barriers
+      // and no wait for the sums (three and one below).  And A_oo^-1 D_oe x = sum a t,
+      // so chi_o is one multiply-add per step instead of one more pass of hops.  With
+      // the loads ahead and the L2 prefetch, a launch on 32^3 x 64 in 8x4x4x4 blocks
+      // went from 0.551 to 0.497 ms, for 12 right-hand sides on 24^3 x 48 from 2.30
+      // to 1.95 ms.
+      // For 16-bit block fields only: the rounding of the first t stays in every later
+      // t and adds up in chi_o.  In FP32 a block solution is then exact to 1.9e-7 with
+      // 4 steps and 7e-7 with 16, with the hops from r to 1.2e-7 and 1.5e-7 (FP64
+      // alike).  Next to the rounding of the fields, 1.9e-4 in FP16 and 1.5e-3 in
+      // bf16 (the same either way to three digits), that is nothing.
+      cpx<T> alpha = {T(0), T(0)};
+      auto advance = [&] {  // with a of the finished step: x, r, chi_o (s_r holds p, s_t holds t)
+        T pr_re, pr_im, pp;
+        sum3_get(pr_re, pr_im, pp, s_red);
+        const T inv = pp > T(0) ? T(1) / pp : T(0);
+        alpha = {pr_re * inv, pr_im * inv};
+        const Half<T> p = s_half(s_r, ns, re, hf), t = s_half(s_t, ns, re, hf);
 #pragma unroll
-      for (int s = 0; s < 2; ++s)
+        for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          x.c[s][c] = cmadd(alpha, r.c[s][c], x.c[s][c]);
-          r.c[s][c] = cmadd(-alpha, p.c[s][c], r.c[s][c]);
-          chi_o.c[s][c] = cmadd(-alpha, t.c[s][c], chi_o.c[s][c]);
-        }
-    };
+          for (int c = 0; c < 3; ++c) {
+            x.c[s][c] = cmadd(alpha, r.c[s][c], x.c[s][c]);
+            r.c[s][c] = cmadd(-alpha, p.c[s][c], r.c[s][c]);
+            chi_o.c[s][c] = cmadd(-alpha, t.c[s][c], chi_o.c[s][c]);
+          }
+      };
 #pragma unroll 1
-    for (int step = 0; step < 2 * a.nmr; ++step) {
-      const int ph = step & 1;
-      if (ph == 0 && step > 0) advance();
-      const int pk2[2] = {ph ? pkE[0] : pkO[0], ph ? pkE[1] : pkO[1]};
-      const Half<T> hq = block_hops<T>(st, ns, ph ? re : ro, ph ? s_t : s_r, pk2, ph ? Vbh : 0, hf, i, np, s_x);
-      Half<T> cl = clover_half(st, ph ? re : ro, hf, ph ? r : hq);
-      if (ph == 0) {
-        if (step > 0) {
-          const Half<T> t = s_half(s_t, ns, re, hf);
+      for (int step = 0; step < 2 * a.nmr; ++step) {
+        const int ph = step & 1;
+        if (ph == 0 && step > 0) advance();
+        const int pk2[2] = {ph ? pkE[0] : pkO[0], ph ? pkE[1] : pkO[1]};
+        const Half<T> hq = block_hops<T>(st, ns, ph ? re : ro, ph ? s_t : s_r, pk2, ph ? Vbh : 0, hf, i, np, s_x);
+        Half<T> cl = clover_half(st, ph ? re : ro, hf, ph ? r : hq);
+        if (ph == 0) {
+          if (step > 0) {
+            const Half<T> t = s_half(s_t, ns, re, hf);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+              for (int c = 0; c < 3; ++c) cl.c[s][c] = cmadd(-alpha, cl.c[s][c], t.c[s][c]);
+          }
+          if (act) s_half_store(s_t, ns, i, hf, cl);
+        } else {
+          const Half<T> p = half_axpy(cl, hq, T(-1));
+          T pr_re = 0, pr_im = 0, pp = 0;
+          if (act) {
+            half_dots(p, r, pr_re, pr_im, pp);
+            s_half_store(s_r, ns, i, hf, p);
+          }
+          sum3_put(pr_re, pr_im, pp, s_red);
+        }
+        __syncthreads();
+      }
+      if (a.nmr > 0) advance();
+    } else {
+      // FP32 and FP64 fields: t from r in every step, and chi_o by one more phase 0, on
+      // x in the place of r (the same code: 24^3 x 48 FP32 in 4^4 blocks 0.272 ms, with
+      // a copy of its own 0.298).
+#pragma unroll 1
+      for (int step = 0; step <= 2 * a.nmr; ++step) {
+        const int ph = step & 1;
+        const bool last = step == 2 * a.nmr;
+        const int pk2[2] = {ph ? pkE[0] : pkO[0], ph ? pkE[1] : pkO[1]};
+        const Half<T> hq = block_hops<T>(st, ns, ph ? re : ro, ph ? s_t : s_r, pk2, ph ? Vbh : 0, hf, i, np, s_x);
+        const Half<T> cl = clover_half(st, ph ? re : ro, hf, last ? half_axpy(rho_o, hq, T(-1)) : (ph ? r : hq));
+        if (last) {
+          chi_o = cl;
+          break;
+        }
+        if (ph == 0) {
+          if (act) s_half_store(s_t, ns, i, hf, cl);
+        } else {
+          const Half<T> p = half_axpy(cl, hq, T(-1));
+          T pr_re = 0, pr_im = 0, pp = 0;
+          if (act) half_dots(p, r, pr_re, pr_im, pp);
+          sum3_put(pr_re, pr_im, pp, s_red);
+          __syncthreads();
+          sum3_get(pr_re, pr_im, pp, s_red);
+          // (a = 0 where |p|^2 has no finite reciprocal: nothing is left to reduce)
+          constexpr T kTiny = sizeof(T) == 4 ? T(1.17549435e-38) : T(2.2250738585072014e-308);
+          const T inv = pp >= kTiny ? T(1) / pp : T(0);
+          const cpx<T> alpha = {pr_re * inv, pr_im * inv};
 #pragma unroll
           for (int s = 0; s < 2; ++s)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) cl.c[s][c] = cmadd(-alpha, cl.c[s][c], t.c[s][c]);
+            for (int c = 0; c < 3; ++c) {
+              x.c[s][c] = cmadd(alpha, r.c[s][c], x.c[s][c]);
+              r.c[s][c] = r.c[s][c] - cmul(alpha, p.c[s][c]);
+            }
+          if (act) s_half_store(s_r, ns, i, hf, step + 1 < 2 * a.nmr ? r : x);
         }
-        if (act) s_half_store(s_t, ns, i, hf, cl);
-      } else {
-        const Half<T> p = half_axpy(cl, hq, T(-1));
-        T pr_re = 0, pr_im = 0, pp = 0;
-        if (act) {
-          half_dots(p, r, pr_re, pr_im, pp);
-          s_half_store(s_r, ns, i, hf, p);
-        }
-        sum3_put(pr_re, pr_im, pp, s_red);
+        __syncthreads();
       }
-      __syncthreads();
     }
-    if (a.nmr > 0) advance();
 
     // ---- outputs: solution, block residual (r on even, 0 on odd), faces
     constexpr int PS = PsiPrec<P>::value;
     typedef typename std::conditional<PS == P64, double, float>::type TS;
     // what the partner needs: chi_o goes to t and chi_e to r (both read for the last
-    // time by their own threads above), the maximum of r to the exchange buffer, into
-    // the slot this thread read last
+    // time by their own threads above; without kLinear r holds chi_e already), the
+    // maximum of r to the exchange buffer, into the slot this thread read last
     T r_max = half_max(r);
     if (act) {
       s_half_store(s_t, ns, i, hf, chi_o);
-      s_half_store(s_r, ns, i, hf, x);
+      if (kLinear) s_half_store(s_r, ns, i, hf, x);
     }
     T* s_m = s_x + Chunk<T>::R * ((12 / Chunk<T>::R) * (1 - hf) * np + i);
     *s_m = r_max;
