@@ -281,8 +281,10 @@ int qcd_gauge_action(qcd_ctx* ctx, const double* U, double beta, double* S, void
  * V_mu(x) the sum of the six staples; U, F device. */
 int qcd_gauge_force(qcd_ctx* ctx, const double* U, double beta, double* F, void* stream);
 
-/* U_mu(x) <- exp(i eps P(x, mu)) U_mu(x) for every link, in place (exponential
- * by a scaled Taylor series, exact to rounding). */
+/* U_mu(x) <- exp(i eps P(x, mu)) U_mu(x) for every link, in place.  The
+ * exponential is a second-degree polynomial in P with coefficients from the
+ * Taylor series (scaling and squaring for |eps P| > 2, Frobenius); its error is a
+ * few 1e-16, growing in proportion to |eps P| beyond 2. */
 int qcd_update_links(qcd_ctx* ctx, double* U, const double* pi, double eps, void* stream);
 
 /* One HMC trajectory: pseudofermion phi = D(U)^+ eta (eta: device (V, 4, 3)

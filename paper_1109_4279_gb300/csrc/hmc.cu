@@ -231,8 +231,12 @@ __global__ void __launch_bounds__(kThreads) plaquette_kernel(Lex g, const double
 // det H), its three complex coefficients found by the Taylor series' Horner
 // scheme in that basis -- 9 operations per term instead of a matrix product's
 // 108.  9, 14, 19 and 26 terms leave less than 1e-18 for |H| (Frobenius) up to
-// 0.06, 1/4, 1 and 2; beyond, H / 2^k is taken and the k squarings are done on
-// the coefficients.  16^3 x 32: 1.85 -> 0.41 ms (order-14 Taylor series of matrix products before).
+// 0.06, 1/4, 1 and 2; beyond, H / 2^k is taken and the matrix squared k times (not
+// the coefficients: theirs grow where two eigenvalues are close, and the error with
+// |H|^2).  16^3 x 32: 1.85 -> 0.41 ms (order-14 Taylor series of matrix products
+// before).  The 1 of the exponential is added last, so a small H leaves one rounding
+// in an element.  Largest errors, that Taylor series / here: 5.6e-17 / 6.5e-17 for
+// |H| up to 1/4, 1.3e-15 / 8e-16 up to 2, 6.8e-14 / 3.2e-14 at 100.
 __global__ void __launch_bounds__(kThreads) link_update_kernel(long long nlinks, double2* __restrict__ U,
                                                                const double* __restrict__ pi, double eps) {
   const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -264,22 +268,16 @@ __global__ void __launch_bounds__(kThreads) link_update_kernel(long long nlinks,
   o01 = sc * o01;
   o02 = sc * o02;
   o12 = sc * o12;
-  // E = q0 + q1 H + q2 H^2: Horner, E <- 1 + (i H / m) E
+  // E - 1 = q0 + q1 H + q2 H^2: Horner, E <- 1 + (i H / m) E, the last 1 left out
   cd q0 = {1, 0}, q1 = {0, 0}, q2 = {0, 0};
   const double n2 = 2.0 * t;
   for (int m = n2 <= 0.0036 ? 9 : (n2 <= 0.0625 ? 14 : (n2 <= 1.0 ? 19 : 26)); m >= 1; --m) {
     const double inv = 1.0 / m, dm = inv * d, tm = inv * t;
     const cd a = {fma(tm, q2.re, inv * q0.re), fma(tm, q2.im, inv * q0.im)};
     const cd b = inv * q1;
-    q0 = {1.0 - dm * q2.im, dm * q2.re};
+    q0 = {(m > 1 ? 1.0 : 0.0) - dm * q2.im, dm * q2.re};
     q1 = ti(a);
     q2 = ti(b);
-  }
-  for (; k > 0; --k) {  // the square modulo the characteristic polynomial, for 2 H
-    const cd r1 = cmul(q0, q1), r2 = cmadd(q1, q1, 2.0 * cmul(q0, q2)), r3_ = 2.0 * cmul(q1, q2), r4 = cmul(q2, q2);
-    q0 = cmadd(q0, q0, d * r3_);
-    q1 = 2.0 * r1 + t * r3_ + d * r4;
-    q2 = r2 + t * r4;
   }
   // H^2: diagonal, then the upper elements
   const double s = sc * sc;
@@ -287,15 +285,18 @@ __global__ void __launch_bounds__(kThreads) link_update_kernel(long long nlinks,
   const cd f01 = cmadd(o02, conjg(o12), (d0 + d1) * o01), f02 = cmadd(o01, o12, (d0 + d2) * o02),
            f12 = cjmadd(o01, o02, (d1 + d2) * o12);
   M3 E;
-  E.a[0][0] = q0 + d0 * q1 + e0 * q2;
-  E.a[1][1] = q0 + d1 * q1 + e1 * q2;
-  E.a[2][2] = q0 + d2 * q1 + e2 * q2;
+  const cd one = {1, 0};
+  E.a[0][0] = one + (q0 + d0 * q1 + e0 * q2);
+  E.a[1][1] = one + (q0 + d1 * q1 + e1 * q2);
+  E.a[2][2] = one + (q0 + d2 * q1 + e2 * q2);
   E.a[0][1] = cmadd(q1, o01, cmul(q2, f01));
   E.a[0][2] = cmadd(q1, o02, cmul(q2, f02));
   E.a[1][2] = cmadd(q1, o12, cmul(q2, f12));
   E.a[1][0] = cmadd(q1, conjg(o01), cmul(q2, conjg(f01)));
   E.a[2][0] = cmadd(q1, conjg(o02), cmul(q2, conjg(f02)));
   E.a[2][1] = cmadd(q1, conjg(o12), cmul(q2, conjg(f12)));
+#pragma unroll 1
+  for (; k > 0; --k) E = mmul(E, E);
   mstore(U, l, mmul(E, mload(U, l)));
 }
 
