@@ -376,13 +376,17 @@ __global__ void __launch_bounds__(128) clover_build_kernel(Geom g, double m0, do
 
 int build_clover(qcd_ctx* c, cudaStream_t s) {
   if (!c->gauge_loaded) return QCD_ERR_STATE;
-  ++c->gen;  // every clover record is reallocated
+  ++c->gen;  // captured graphs hold the records of the last build
+  // After qcd_load_gauge the FP64 records are written again in place: nothing can still
+  // be reading them, or it would be reading links that the load replaced.  A term built
+  // a second time on the same links may have readers queued on any stream, so all its
+  // records are freed, which waits for them, and allocated anew.  (Not
+  // cudaDeviceSynchronize: that fails while another thread captures a stream, and
+  // contexts are independent.)
+  const bool keep = !c->clover_built;
   c->clover_built = false;  // A's memory is scratch until the last pass
-  // work still queued on other streams may read the records that are kept (the
-  // memory that is freed waits by itself)
-  QCD_CUDA(cudaDeviceSynchronize());
   for (int p = 0; p < 5; ++p) {
-    if (p == P64 && c->A[p].data && c->Ahat[p].data) continue;  // a new gauge field: the same sizes again
+    if (keep && p == P64 && c->A[p].data && c->Ahat[p].data) continue;
     rec_free(c->A[p]);
     rec_free(c->Ahat[p]);
   }

@@ -1,0 +1,77 @@
+"""Contexts are independent: what one thread does with its context does not depend on
+another thread that is capturing a CUDA graph at the same time (thread-local mode).
+"""
+import threading
+
+import pytest
+
+from paper_1109_4279_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+class _Capturing(threading.Thread):
+    """Captures one addition on a stream of its own; stays in capture between
+    `begun` and `finish`."""
+
+    def __init__(self):
+        super().__init__()
+        self.begun, self.finish = threading.Event(), threading.Event()
+        self.x = torch.ones(256, device="cuda")
+        self.y = torch.zeros(256, device="cuda")
+        self.graph = torch.cuda.CUDAGraph()
+        self.error = None
+
+    def run(self):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                torch.add(self.x, 1.0, out=self.y)
+                torch.cuda.synchronize()
+                self.graph.capture_begin(capture_error_mode="thread_local")
+                torch.add(self.x, 2.0, out=self.y)
+                self.begun.set()
+                self.finish.wait(60)
+                self.graph.capture_end()
+        except Exception as e:  # (reported by the main thread)
+            self.error = e
+        finally:
+            self.begun.set()
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        self.start()
+        assert self.begun.wait(60)
+        return self
+
+    def __exit__(self, *exc):
+        self.finish.set()
+        self.join()
+        if exc[0] is None:
+            assert self.error is None
+            self.graph.replay()
+            torch.cuda.synchronize()
+            assert bool((self.y == 3.0).all())
+
+
+def test_clover_rebuild_while_another_thread_captures():
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (4, 4, 4, 8), (2, 2, 2, 2)
+    fields = [synth.gauge_field(dims, 0.5, k)[0] for k in (51, 52)]
+    Us = [torch.from_numpy(U).cuda() for U in fields]
+    psi = torch.from_numpy(synth.gaussian_spinor(dims, synth.gauge_field(dims, 0.5, 53)[1])).cuda()
+    outs = [torch.empty_like(psi) for _ in range(4)]
+    lat = B.Lattice(dims, block, 0.1, 1.3)
+    lat.load_gauge(Us[0])
+    with _Capturing():
+        lat.load_gauge(Us[1])        # new links: the FP64 records are used again
+        B.qcd_apply_D(lat.ctx, psi, outs[0])
+        B.qcd_build_clover(lat.ctx)  # the same links once more
+        B.qcd_apply_D(lat.ctx, psi, outs[1])
+    for k, U in enumerate(Us):
+        fresh = B.Lattice(dims, block, 0.1, 1.3)
+        fresh.load_gauge(U)
+        B.qcd_apply_D(fresh.ctx, psi, outs[2 + k])
+        fresh.close()
+    assert torch.equal(outs[0], outs[3]) and torch.equal(outs[1], outs[3]) and not torch.equal(outs[2], outs[3])
+    lat.close()
