@@ -23,13 +23,13 @@ void cg_release(Workspace& w) {
   w.h_cg = nullptr;
 }
 
-static int cg_prepare(qcd_ctx* c, Workspace& w, size_t nvec = 4) {
+static int cg_prepare(qcd_ctx* c, Workspace& w, cudaStream_t s, size_t nvec = 4) {
   if (!w.r.data) QCD_TRY(rec_alloc(w.r, P64, 24, c->V));
   while (w.cgv.size() < nvec) {
     w.cgv.emplace_back();
     QCD_TRY(rec_alloc(w.cgv.back(), P64, 24, c->V));
   }
-  if (!w.d_part) QCD_TRY(partials_alloc(c->V, 1, &w.d_part, &w.ps));
+  if (!w.d_part) QCD_TRY(partials_alloc(c->V, 1, &w.d_part, &w.ps, s));
   if (!w.d_cg) QCD_CUDA(cudaMalloc(&w.d_cg, sizeof(double) * 8));
   if (!w.h_cg) QCD_CUDA(cudaMallocHost(&w.h_cg, sizeof(double) * 8));
   return QCD_OK;
@@ -45,7 +45,7 @@ static int cg_solve(Problem& p, const qcd_solver_params& sp, bool fallback) {
   const size_t dsz = sizeof(double);
   if (!fallback) memset(&p.info, 0, sizeof(p.info));
   p.status = QCD_OK;
-  QCD_TRY(cg_prepare(c, w));
+  QCD_TRY(cg_prepare(c, w, s));
   Rec& R = w.cgv[0];
   Rec& P = w.cgv[1];
   Rec& T = w.cgv[2];
@@ -128,7 +128,7 @@ static int cg_eo_solve(Problem& p, const qcd_solver_params& sp, bool fallback) {
   const size_t dsz = sizeof(double);
   if (!fallback) memset(&p.info, 0, sizeof(p.info));
   p.status = QCD_OK;
-  QCD_TRY(cg_prepare(c, w, 6));
+  QCD_TRY(cg_prepare(c, w, s, 6));
   Rec& R = w.cgv[0];
   Rec& P = w.cgv[1];
   Rec& T = w.cgv[2];

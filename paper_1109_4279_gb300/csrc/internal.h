@@ -384,8 +384,10 @@ int reduce_partials(const double* partials, int nparts, int stride, int m, doubl
 
 // ---- solver.cu
 size_t partials_for(long long V);
-// allocate nr right-hand sides' partial sums (*ps doubles each), their heads cleared
-int partials_alloc(long long V, int nr, double** part, long long* ps);
+// allocate nr right-hand sides' partial sums (*ps doubles each), their heads cleared on
+// s (not on the default stream: that fails while another thread captures one that waits
+// for it)
+int partials_alloc(long long V, int nr, double** part, long long* ps, cudaStream_t s);
 // allocate the solver fields and scalars of nr right-hand sides (a change of
 // nr reallocates everything)
 int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream_t s, int nr = 1);

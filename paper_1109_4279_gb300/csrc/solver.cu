@@ -46,17 +46,20 @@ size_t partials_for(long long V) {
   return kPartHead + (blas > resid ? blas : resid);
 }
 
-int partials_alloc(long long V, int nr, double** part, long long* ps) {
+int partials_alloc(long long V, int nr, double** part, long long* ps, cudaStream_t s) {
   const size_t n = partials_for(V);
   if (cudaMalloc(part, sizeof(double) * n * nr) != cudaSuccess) {
     cudaGetLastError();
     *part = nullptr;
     return QCD_ERR_NOMEM;
   }
+  const cudaError_t e = cudaMemset2DAsync(*part, sizeof(double) * n, 0, sizeof(double) * kPartHead, nr, s);
+  if (e != cudaSuccess) {  // sums counted from an uncleared head would be wrong
+    cudaFree(*part);
+    *part = nullptr;
+    return cuda_fail(e, "partials_alloc");
+  }
   *ps = (long long)n;
-  // (the solver's streams do not wait for the default stream by themselves)
-  QCD_CUDA(cudaMemset2DAsync(*part, sizeof(double) * n, 0, sizeof(double) * kPartHead, nr, nullptr));
-  QCD_CUDA(cudaStreamSynchronize(nullptr));
   return QCD_OK;
 }
 
@@ -137,7 +140,7 @@ int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream
     w.pprec = pprec;
   }
   if (!w.rho.data) QCD_TRY(rec_alloc(w.rho, rprec, 24, Vn));
-  if (!w.d_part) QCD_TRY(partials_alloc(c->V, nr, &w.d_part, &w.ps));
+  if (!w.d_part) QCD_TRY(partials_alloc(c->V, nr, &w.d_part, &w.ps, s));
   if (nkv > w.nkv) {
     graphs_clear(w);
     for (int k = w.nkv; k < nkv; ++k) {

@@ -1,6 +1,7 @@
 """Contexts are independent: what one thread does with its context does not depend on
 another thread that is capturing a CUDA graph at the same time (thread-local mode).
 """
+import ctypes
 import threading
 
 import pytest
@@ -15,8 +16,14 @@ class _Capturing(threading.Thread):
     """Captures one addition on a stream of its own; stays in capture between
     `begun` and `finish`."""
 
-    def __init__(self):
+    def __init__(self, blocking=False):
         super().__init__()
+        if blocking:  # a stream that waits for the legacy default stream
+            handle = ctypes.c_void_p()
+            assert int(torch.cuda.cudart().cudaStreamCreate(ctypes.addressof(handle))) == 0
+            self.stream = torch.cuda.ExternalStream(handle.value)
+        else:
+            self.stream = torch.cuda.Stream()
         self.begun, self.finish = threading.Event(), threading.Event()
         self.x = torch.ones(256, device="cuda")
         self.y = torch.zeros(256, device="cuda")
@@ -25,7 +32,7 @@ class _Capturing(threading.Thread):
 
     def run(self):
         try:
-            with torch.cuda.stream(torch.cuda.Stream()):
+            with torch.cuda.stream(self.stream):
                 torch.add(self.x, 1.0, out=self.y)
                 torch.cuda.synchronize()
                 self.graph.capture_begin(capture_error_mode="thread_local")
@@ -75,3 +82,30 @@ def test_clover_rebuild_while_another_thread_captures():
         fresh.close()
     assert torch.equal(outs[0], outs[3]) and torch.equal(outs[1], outs[3]) and not torch.equal(outs[2], outs[3])
     lat.close()
+
+
+def test_first_solve_while_another_thread_captures_a_blocking_stream():
+    """The first solve of a context allocates its workspace; nothing of that may go
+    through the default stream, which the captured stream waits for."""
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (4, 4, 4, 8), (2, 2, 2, 2)
+    U, rng = synth.gauge_field(dims, 0.5, 54)
+    U = torch.from_numpy(U).cuda()
+    b = torch.from_numpy(synth.gaussian_spinor(dims, rng)).cuda()
+    sp = B.solver_params(tol=1e-10, solver="cg")
+    xs = [torch.zeros_like(b) for _ in range(3)]
+    contexts = [B.Lattice(dims, block, 0.1, 1.3) for _ in range(2)]
+    for lat in contexts:
+        lat.load_gauge(U)
+    _, want = B.qcd_solve(contexts[0].ctx, b, xs[0], 1, sp)
+    side = torch.cuda.Stream()
+    with _Capturing(blocking=True):
+        with torch.cuda.stream(side):
+            st, _ = B.qcd_solve(contexts[1].ctx, b, xs[1], 1, sp, raise_on_fail=False)
+    torch.cuda.synchronize()
+    assert st == 0
+    _, info = B.qcd_solve(contexts[1].ctx, b, xs[2], 1, sp)
+    assert info[0]["cg_iterations"] == want[0]["cg_iterations"]
+    assert torch.equal(xs[1], xs[0]) and torch.equal(xs[2], xs[0])
+    for lat in contexts:
+        lat.close()
