@@ -156,8 +156,12 @@ void qcd_solver_defaults(qcd_solver_params* sp);
  * chessboard colouring additionally needs an even number of blocks per
  * direction, and the even/odd split inside blocks even block extents),
  * uploads the layout tables and returns *out (caller frees with qcd_destroy).
- * Device memory for fields is allocated on first use.  Errors: QCD_ERR_ARG,
- * QCD_ERR_GEOMETRY, QCD_ERR_CUDA, QCD_ERR_NOMEM.
+ * Device memory for fields is allocated on first use.  qcd_apply_D, qcd_force and
+ * qcd_gradient keep their staging memory for the next call: up to 1 GiB of spinor
+ * fields and 1 GiB of force scratch per context, 2 GiB in all contexts of the
+ * process.  It is given back by qcd_destroy, and when any allocation of the library
+ * finds the device full.  Errors: QCD_ERR_ARG, QCD_ERR_GEOMETRY, QCD_ERR_CUDA,
+ * QCD_ERR_NOMEM.
  */
 int qcd_create(qcd_ctx** out, const qcd_params* p);
 
@@ -439,11 +443,16 @@ int qcd_sap_apply_n(qcd_ctx* ctx, const double* eta, double* psi, int nrhs, int 
  *                              1 .. 2^31 (default 2^31);
  *   QCD_DEBUG_SAP_EXTRA_TX:    bytes the staging barrier expects beyond the
  *                              copies, 0 .. 4096 (default 0; any other value
- *                              makes every wait run out).
+ *                              makes every wait run out);
+ *   QCD_DEBUG_ALLOC_LIMIT:     (of the calling thread, every context) a device
+ *                              allocation that would take the staging memory kept
+ *                              by all contexts plus itself beyond this many bytes
+ *                              fails as on a full device (default 0: none does).
  * Returns QCD_ERR_ARG for an unknown setting or a value out of range.
  */
 #define QCD_DEBUG_SAP_WAIT_CYCLES 0
 #define QCD_DEBUG_SAP_EXTRA_TX 1
+#define QCD_DEBUG_ALLOC_LIMIT 2
 int qcd_debug_set(qcd_ctx* ctx, int what, long long value);
 
 /*

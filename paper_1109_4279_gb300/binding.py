@@ -365,11 +365,11 @@ def qcd_get_sap_tile(ctx, nrhs):
     return rt
 
 
-DEBUG = {"sap_wait_cycles": 0, "sap_extra_tx": 1}
+DEBUG = {"sap_wait_cycles": 0, "sap_extra_tx": 1, "alloc_limit": 2}
 
 
 def qcd_debug_set(ctx, what, value):
-    """Test hooks of the SAP staging wait (see include/qcdgb.h)."""
+    """Test hooks of the SAP staging wait and of device allocation (see include/qcdgb.h)."""
     return check(lib().qcd_debug_set(ctx, DEBUG[what] if isinstance(what, str) else int(what), int(value)),
                  "qcd_debug_set")
 

@@ -2,6 +2,7 @@
 // staging, context lifetime and kernel instrumentation.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -22,7 +23,7 @@ int rec_alloc(Rec& r, int prec, int nreal, long long V) {
   const size_t data = (size_t)V * chunks(prec, nreal) * 16;
   const size_t norm = (prec == P16 || prec == PB16) ? (size_t)V * sizeof(float) : 0;
   void* p = nullptr;
-  if (cudaMalloc(&p, data + norm) != cudaSuccess) {
+  if (dev_malloc(&p, data + norm) != cudaSuccess) {
     cudaGetLastError();
     return QCD_ERR_NOMEM;
   }
@@ -49,13 +50,61 @@ Rec rec_view(void* p, int prec, int nreal, long long V) {
   return r;
 }
 
-// frees the kept buffer of a slot that no call holds
-static void scratch_drop(qcd_ctx* c, int slot) {
-  if (c->scratch_busy[slot].exchange(1)) return;
+// the contexts that exist, and the bytes that all of them keep in their slots
+static std::mutex g_ctx_mutex;
+static qcd_ctx* g_ctx_list = nullptr;
+static std::atomic<size_t> g_kept{0};
+static thread_local size_t t_alloc_limit = 0;  // test hook (QCD_DEBUG_ALLOC_LIMIT), 0: none
+
+static void ctx_register(qcd_ctx* c) {
+  std::lock_guard<std::mutex> lock(g_ctx_mutex);
+  c->next = g_ctx_list;
+  g_ctx_list = c;
+}
+
+static void ctx_unregister(qcd_ctx* c) {
+  std::lock_guard<std::mutex> lock(g_ctx_mutex);
+  for (qcd_ctx** p = &g_ctx_list; *p; p = &(*p)->next)
+    if (*p == c) {
+      *p = c->next;
+      return;
+    }
+}
+
+// frees what a slot keeps (the caller holds the slot)
+static void scratch_free(qcd_ctx* c, int slot) {
   if (c->scratch[slot]) cudaFree(c->scratch[slot]);
+  g_kept -= c->scratch_bytes[slot];
   c->scratch[slot] = nullptr;
   c->scratch_bytes[slot] = 0;
-  c->scratch_busy[slot].store(0);
+}
+
+// gives back what the contexts keep and no call holds
+static void scratch_trim() {
+  std::lock_guard<std::mutex> lock(g_ctx_mutex);
+  for (qcd_ctx* c = g_ctx_list; c; c = c->next)
+    for (int k = 0; k < kScratchSlots; ++k)
+      if (!c->scratch_busy[k].exchange(1)) {
+        scratch_free(c, k);
+        c->scratch_busy[k].store(0);
+      }
+}
+
+static cudaError_t malloc_once(void** p, size_t bytes) {
+  if (t_alloc_limit && bytes + g_kept.load() > t_alloc_limit) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
+cudaError_t dev_malloc_bytes(void** p, size_t bytes) {
+  *p = nullptr;
+  cudaError_t e = malloc_once(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    scratch_trim();
+    e = malloc_once(p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
 }
 
 int Scratch::get(qcd_ctx* c, int slot_, size_t bytes) {
@@ -66,25 +115,21 @@ int Scratch::get(qcd_ctx* c, int slot_, size_t bytes) {
       p = c->scratch[slot];
       return QCD_OK;
     }
-    if (c->scratch[slot]) cudaFree(c->scratch[slot]);
-    c->scratch[slot] = nullptr;
-    c->scratch_bytes[slot] = 0;
+    scratch_free(c, slot);
   }
-  cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {  // once more without what the context keeps
+  if (dev_malloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
-    for (int k = 0; k < kScratchSlots; ++k) scratch_drop(c, k);
-    e = cudaMalloc(&p, bytes);
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
     return QCD_ERR_NOMEM;
   }
-  own = !claimed;
+  own = true;
   if (claimed) {
-    c->scratch[slot] = p;
-    c->scratch_bytes[slot] = bytes;
+    if (g_kept.fetch_add(bytes) + bytes <= kScratchKeepAll) {
+      own = false;
+      c->scratch[slot] = p;
+      c->scratch_bytes[slot] = bytes;
+    } else {
+      g_kept -= bytes;
+    }
   }
   return QCD_OK;
 }
@@ -211,7 +256,7 @@ int qcd_create(qcd_ctx** out, const qcd_params* p) {
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   if (st == QCD_OK) {
-    if (cudaMalloc(&c->d_scalars, 64 * 1024) != cudaSuccess || cudaMallocHost(&c->h_scalars, 64 * 1024) != cudaSuccess ||
+    if (dev_malloc(&c->d_scalars, 64 * 1024) != cudaSuccess || cudaMallocHost(&c->h_scalars, 64 * 1024) != cudaSuccess ||
         cudaMemset(c->d_scalars, 0, 64 * 1024) != cudaSuccess)
       st = QCD_ERR_NOMEM;
   }
@@ -219,12 +264,14 @@ int qcd_create(qcd_ctx** out, const qcd_params* p) {
     qcd_destroy(c);
     return st;
   }
+  ctx_register(c);
   *out = c;
   return QCD_OK;
 }
 
 void qcd_destroy(qcd_ctx* c) {
   if (!c) return;
+  ctx_unregister(c);
   cudaDeviceSynchronize();
   workspace_free(c);
   for (int p = 0; p < 5; ++p) {
@@ -236,8 +283,7 @@ void qcd_destroy(qcd_ctx* c) {
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
   if (c->deliver_stream) cudaStreamDestroy(c->deliver_stream);
   c->streams.clear();
-  for (void* p : c->scratch)
-    if (p) cudaFree(p);
+  for (int k = 0; k < kScratchSlots; ++k) scratch_free(c, k);
   if (c->d_tables) cudaFree(c->d_tables);
   if (c->d_scalars) cudaFree(c->d_scalars);
   if (c->h_scalars) cudaFreeHost(c->h_scalars);
@@ -256,7 +302,7 @@ int qcd_load_gauge(qcd_ctx* c, const double* U, int is_device, void* stream) {
   const size_t bytes = (size_t)c->V * 4 * 9 * 16;
   if (is_device) return load_gauge_device(c, U, s);
   void* tmp = nullptr;
-  if (cudaMalloc(&tmp, bytes) != cudaSuccess) {
+  if (dev_malloc(&tmp, bytes) != cudaSuccess) {
     cudaGetLastError();
     return QCD_ERR_NOMEM;
   }
@@ -359,7 +405,7 @@ static int solve_problems(std::vector<Problem>& probs, const double* const* b, d
         if (w.stage) cudaFree(w.stage);
         w.stage = nullptr;
         w.stage_bytes = 0;
-        if (cudaMalloc(&w.stage, 2 * fbytes) != cudaSuccess) {
+        if (dev_malloc(&w.stage, 2 * fbytes) != cudaSuccess) {
           cudaGetLastError();
           w.stage = nullptr;
           st = QCD_ERR_NOMEM;
@@ -442,7 +488,7 @@ static int solve_tile(qcd_ctx* c, const double* b, double* x, int nrhs, bool dev
       if (w->stage) cudaFree(w->stage);
       w->stage = nullptr;
       w->stage_bytes = 0;
-      if (cudaMalloc(&w->stage, 2 * fbytes) != cudaSuccess) {
+      if (dev_malloc(&w->stage, 2 * fbytes) != cudaSuccess) {
         cudaGetLastError();
         w->stage = nullptr;
         return QCD_ERR_NOMEM;
@@ -793,6 +839,10 @@ int qcd_debug_set(qcd_ctx* c, int what, long long value) {
     case QCD_DEBUG_SAP_EXTRA_TX:
       if (value < 0 || value > 4096) return QCD_ERR_ARG;
       c->dbg_sap_extra_tx = (int)value;
+      return QCD_OK;
+    case QCD_DEBUG_ALLOC_LIMIT:
+      if (value < 0) return QCD_ERR_ARG;
+      t_alloc_limit = (size_t)value;
       return QCD_OK;
     default:
       return QCD_ERR_ARG;

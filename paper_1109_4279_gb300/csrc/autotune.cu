@@ -235,9 +235,9 @@ extern "C" int qcd_tune_block(const qcd_params* p, const double* U, const double
   double* db = nullptr;
   double* dU = nullptr;
   int st = QCD_OK;
-  if (cudaMalloc(&dx, fbytes) != cudaSuccess) st = QCD_ERR_NOMEM;
+  if (dev_malloc(&dx, fbytes) != cudaSuccess) st = QCD_ERR_NOMEM;
   if (st == QCD_OK && !is_device) {
-    if (cudaMalloc(&db, fbytes) != cudaSuccess || cudaMalloc(&dU, (size_t)V * 4 * 9 * 16) != cudaSuccess)
+    if (dev_malloc(&db, fbytes) != cudaSuccess || dev_malloc(&dU, (size_t)V * 4 * 9 * 16) != cudaSuccess)
       st = QCD_ERR_NOMEM;
     if (st == QCD_OK) {
       cudaMemcpy(db, b, fbytes, cudaMemcpyHostToDevice);

@@ -30,7 +30,7 @@ static int cg_prepare(qcd_ctx* c, Workspace& w, cudaStream_t s, size_t nvec = 4)
     QCD_TRY(rec_alloc(w.cgv.back(), P64, 24, c->V));
   }
   if (!w.d_part) QCD_TRY(partials_alloc(c->V, 1, &w.d_part, &w.ps, s));
-  if (!w.d_cg) QCD_CUDA(cudaMalloc(&w.d_cg, sizeof(double) * 8));
+  if (!w.d_cg) QCD_CUDA(dev_malloc(&w.d_cg, sizeof(double) * 8));
   if (!w.h_cg) QCD_CUDA(cudaMallocHost(&w.h_cg, sizeof(double) * 8));
   return QCD_OK;
 }

@@ -54,7 +54,7 @@ static int dr_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cud
   // pinned column buffer: pass-1 and pass-2 coefficients (2 x 2 (m + 1)) and
   // the subdiagonal; device buffer: subdiagonals, then restart coefficients
   if (!w.h_hcol) QCD_CUDA(cudaMallocHost(&w.h_hcol, sizeof(double) * (4 * 65 + 8)));
-  if (!w.d_hnorm) QCD_CUDA(cudaMalloc(&w.d_hnorm, sizeof(double) * (65 + 2 * 65 * 65)));
+  if (!w.d_hnorm) QCD_CUDA(dev_malloc(&w.d_hnorm, sizeof(double) * (65 + 2 * 65 * 65)));
   return QCD_OK;
 }
 

@@ -343,7 +343,7 @@ struct HmcScratch {
   }
   int init(long long V) {
     nparts = grid_for(V * 4);
-    if (cudaMalloc(&part, sizeof(double) * nparts) != cudaSuccess || cudaMalloc(&res, sizeof(double)) != cudaSuccess) {
+    if (dev_malloc(&part, sizeof(double) * nparts) != cudaSuccess || dev_malloc(&res, sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       return QCD_ERR_NOMEM;
     }
@@ -424,7 +424,7 @@ struct DevBuf {
     if (p) cudaFree(p);
   }
   int alloc(size_t n) {
-    if (cudaMalloc(&p, n * sizeof(double)) != cudaSuccess) {
+    if (dev_malloc(&p, n * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
       return QCD_ERR_NOMEM;

@@ -195,6 +195,7 @@ struct qcd_ctx {
   void* scratch[2] = {nullptr, nullptr};  // kept staging buffers (qcd::Scratch)
   size_t scratch_bytes[2] = {0, 0};
   std::atomic<int> scratch_busy[2] = {{0}, {0}};  // a call holds the slot
+  qcd_ctx* next = nullptr;  // list of the process's contexts
   double* d_scalars = nullptr;  // small device array for coefficients
   double* h_scalars = nullptr;  // pinned host mirror
   // test hooks (qcd_debug_set): budget of the SAP staging wait, and bytes its
@@ -231,14 +232,26 @@ struct ProfScope {
 };
 
 // ---- memory helpers (api.cu)
+// cudaMalloc for every allocation of the library: when the device has no room, what the
+// contexts keep for later calls (qcd::Scratch) is given back and the request made once
+// more, so that kept memory never makes a call fail.
+cudaError_t dev_malloc_bytes(void** p, size_t bytes);
+template <typename T>
+cudaError_t dev_malloc(T** p, size_t bytes) {
+  void* q = nullptr;
+  const cudaError_t e = dev_malloc_bytes(&q, bytes);
+  *p = (T*)q;
+  return e;
+}
 // Staging memory of a context for entry points that need fields or scratch only
 // while they run (cudaMalloc and cudaFree took 100 to 300 us of each such call).
 // A slot's buffer of up to kScratchKeep bytes is kept for the next call.  A call
 // claims the slot until it returns, and every such entry point waits for its work
 // before that, so calls on different streams never share the buffer; a call that
 // finds the slot claimed (another thread's) and one that wants more allocates and
-// frees its own.  Freed with the context, or when an allocation here fails.
-static constexpr size_t kScratchKeep = (size_t)1 << 30;
+// frees its own.  All contexts of the process together keep kScratchKeepAll bytes at
+// most; it is freed with the context, or by dev_malloc when the device is full.
+static constexpr size_t kScratchKeep = (size_t)1 << 30, kScratchKeepAll = (size_t)2 << 30;
 struct Scratch {
   void* p = nullptr;
   bool own = false;           // allocated for this call alone

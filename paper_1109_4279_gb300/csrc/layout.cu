@@ -55,7 +55,7 @@ int setup_geometry(qcd_ctx* c) {
     j2r[j] = r;
     r2y[r] = y[0] | (y[1] << 8) | (y[2] << 16) | (y[3] << 24);
   }
-  QCD_CUDA(cudaMalloc(&c->d_tables, sizeof(int) * 2 * Vb));
+  QCD_CUDA(dev_malloc(&c->d_tables, sizeof(int) * 2 * Vb));
   QCD_CUDA(cudaMemcpy(c->d_tables, tab.data(), sizeof(int) * 2 * Vb, cudaMemcpyHostToDevice));
   g.r2y = c->d_tables;
   g.j2r = c->d_tables + Vb;
@@ -301,7 +301,7 @@ int load_gauge_device(qcd_ctx* c, const double* lex_dev, cudaStream_t s) {
   ++c->gen;  // the links change (and their reduced-precision copies are freed)
   if (!c->U[P64]) {
     c->U_bytes[P64] = (size_t)c->V * GaugeLayout<P64>::bytes_per_site;
-    if (cudaMalloc(&c->U[P64], c->U_bytes[P64]) != cudaSuccess) {
+    if (dev_malloc(&c->U[P64], c->U_bytes[P64]) != cudaSuccess) {
       c->U[P64] = nullptr;
       return QCD_ERR_NOMEM;
     }
@@ -373,7 +373,7 @@ int ensure_gauge(qcd_ctx* c, int prec, cudaStream_t s) {
   size_t bytes = (size_t)c->V * ((prec == P64 || prec == PDF) ? GaugeLayout<P64>::bytes_per_site
                                  : (prec == P32 ? GaugeLayout<P32>::bytes_per_site
                                                 : GaugeLayout<P16>::bytes_per_site));
-  if (cudaMalloc(&c->U[prec], bytes) != cudaSuccess) {
+  if (dev_malloc(&c->U[prec], bytes) != cudaSuccess) {
     c->U[prec] = nullptr;
     return QCD_ERR_NOMEM;
   }

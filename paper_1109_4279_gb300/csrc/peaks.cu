@@ -66,7 +66,7 @@ static int time_peak(int lanes_per_elem, int iters, double* tflops, cudaStream_t
   QCD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int grid = sms * 8;
   float* sink = nullptr;
-  QCD_CUDA(cudaMalloc(&sink, sizeof(float) * grid));
+  QCD_CUDA(dev_malloc(&sink, sizeof(float) * grid));
   // a and b keep the chains bounded: x -> 0.999 x + 1e-3 converges to 1
   fma_peak_kernel<T><<<grid, kPeakThreads, 0, s>>>(iters / 8, 0.999f, 1e-3f, sink);  // warm-up (clock ramp)
   QCD_LAUNCHED();

@@ -1427,7 +1427,7 @@ int sap_prepare(qcd_ctx* c, SapWork& w, int prec, cudaStream_t s, int nr) {
   int F = 0;
   for (int mu = 0; mu < 4; ++mu) F += 2 * (g.Vb / g.b[mu]);
   w.faces_bytes = (size_t)c->nblk * F * 12 * (dbl ? 8 : 4) * nr;
-  if (cudaMalloc(&w.faces, w.faces_bytes) != cudaSuccess) {
+  if (dev_malloc(&w.faces, w.faces_bytes) != cudaSuccess) {
     cudaGetLastError();
     w.faces = nullptr;
     return QCD_ERR_NOMEM;

@@ -48,7 +48,7 @@ size_t partials_for(long long V) {
 
 int partials_alloc(long long V, int nr, double** part, long long* ps, cudaStream_t s) {
   const size_t n = partials_for(V);
-  if (cudaMalloc(part, sizeof(double) * n * nr) != cudaSuccess) {
+  if (dev_malloc(part, sizeof(double) * n * nr) != cudaSuccess) {
     cudaGetLastError();
     *part = nullptr;
     return QCD_ERR_NOMEM;
@@ -153,7 +153,7 @@ int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream
     // one block of scalars per right-hand side: a1, a2 (2 nkv^2 each), cr (3 nkv),
     // rn (nkv + 8), gam (2 nkv), gs (8 nkv)
     const long long ss = 4LL * nkv * nkv + 3 * nkv + (nkv + 8) + 2 * nkv + 8 * nkv;
-    QCD_CUDA(cudaMalloc(&w.d_scal, sizeof(double) * ss * nr));
+    QCD_CUDA(dev_malloc(&w.d_scal, sizeof(double) * ss * nr));
     QCD_CUDA(cudaMemset(w.d_scal, 0, sizeof(double) * ss * nr));
     w.ss = ss;
     w.d_a1 = w.d_scal;
@@ -163,7 +163,7 @@ int ws_prepare(qcd_ctx* c, Workspace& w, const qcd_solver_params& sp, cudaStream
     w.d_gam = w.d_rn + nkv + 8;
     w.d_gs = w.d_gam + 2 * nkv;
     QCD_CUDA(cudaMallocHost(&w.h_pin, sizeof(double) * (nkv + 8) * nr));
-    QCD_CUDA(cudaMalloc(&w.d_mask, sizeof(int) * 2 * nr));
+    QCD_CUDA(dev_malloc(&w.d_mask, sizeof(int) * 2 * nr));
     QCD_CUDA(cudaMallocHost(&w.h_mask, sizeof(int) * 2 * nr));
     w.d_k = w.d_mask + nr;
     w.h_k = w.h_mask + nr;

@@ -1,0 +1,101 @@
+"""Memory that contexts keep between calls does not make other calls fail: it is
+given back when an allocation finds the device full (a full device is played by the
+library's allocation limit), and all contexts together keep a bounded amount.
+"""
+import contextlib
+
+import pytest
+
+from paper_1109_4279_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+NOMEM = -4
+
+
+@contextlib.contextmanager
+def _limit(lat, n):
+    from paper_1109_4279_gb300 import binding as B
+    B.qcd_debug_set(lat.ctx, "alloc_limit", n)
+    try:
+        yield
+    finally:
+        B.qcd_debug_set(lat.ctx, "alloc_limit", 0)
+
+
+def _lattices(n, dims, block, seed):
+    from paper_1109_4279_gb300 import binding as B
+    U, rng = synth.gauge_field(dims, 0.4, seed)
+    lats = [B.Lattice(dims, block, 0.2, 1.1) for _ in range(n)]
+    for lat in lats:
+        lat.load_gauge(torch.from_numpy(U).cuda())
+    return lats, rng
+
+
+@pytest.mark.parametrize("other", [False, True], ids=["same context", "another context"])
+def test_kept_memory_is_given_back(other):
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (16, 16, 16, 16), (4, 4, 4, 4)  # a field of FP64 spinors: 12.6 MB
+    (a, c), rng = _lattices(2, dims, block, 61)
+    b = torch.from_numpy(synth.gaussian_spinor(dims, rng)).cuda()
+    x, y = torch.zeros_like(b), torch.empty_like(b)
+    B.qcd_apply_D(a.ctx, b, y)  # keeps two fields
+    user = c if other else a
+    # the largest allocation of the solve is 18.9 MB (FP32 clover records); with 25.2 MB
+    # kept, its first field does not fit any more
+    with _limit(user, 35_000_000):
+        st, _ = B.qcd_solve(user.ctx, b, x, 1, B.solver_params(tol=1e-10), raise_on_fail=False)
+    assert st == 0
+    want = torch.zeros_like(b)
+    fresh = _lattices(1, dims, block, 61)[0][0]
+    B.qcd_solve(fresh.ctx, b, want, 1, B.solver_params(tol=1e-10))
+    assert torch.equal(x, want)
+    y2 = torch.empty_like(b)
+    B.qcd_apply_D(a.ctx, b, y2)
+    assert torch.equal(y, y2)
+    for lat in (a, c, fresh):
+        lat.close()
+
+
+def test_a_device_that_stays_full():
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (8, 8, 8, 8), (4, 4, 4, 4)
+    (lat,), rng = _lattices(1, dims, block, 62)
+    b = torch.from_numpy(synth.gaussian_spinor(dims, rng)).cuda()
+    x = torch.zeros_like(b)
+    with _limit(lat, 100_000):
+        assert B.lib().qcd_apply_D(lat.ctx, B._ptr(b), B._ptr(x), 0, 0, 1, B._stream()) == NOMEM
+        st, _ = B.qcd_solve(lat.ctx, b, x, 1, B.solver_params(tol=1e-10), raise_on_fail=False)
+        assert st == NOMEM
+    st, info = B.qcd_solve(lat.ctx, b, x, 1, B.solver_params(tol=1e-10))
+    assert st == 0 and info[0]["true_residual"] <= 1e-10
+    lat.close()
+
+
+def test_all_contexts_keep_two_gib_at_most():
+    """Each of three contexts stages 1.02 GB for four FP64 right-hand sides."""
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (48, 24, 24, 24), (4, 4, 4, 4)
+    V = 48 * 24 ** 3
+    U = torch.eye(3, dtype=torch.complex128, device="cuda").expand(V, 4, 3, 3).contiguous()
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    psi = torch.view_as_complex(torch.randn((4, V, 4, 3, 2), dtype=torch.float64, device="cuda", generator=gen))
+    outs = [torch.empty_like(psi) for _ in range(4)]
+    lats = [B.Lattice(dims, block, 0.0, 1.0) for _ in range(3)]
+    for lat in lats:
+        lat.load_gauge(U)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for lat, out in zip(lats, outs):
+        B.qcd_apply_D(lat.ctx, psi, out, nrhs=4)
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert 2 * 1.0e9 < kept <= 2 << 30
+    for out in outs[1:3]:
+        assert torch.equal(out, outs[0])
+    lats[0].close()  # its share is free again, and the next call of another context keeps it
+    B.qcd_apply_D(lats[2].ctx, psi, outs[3], nrhs=4)
+    assert torch.equal(outs[3], outs[0])
+    for lat in lats[1:]:
+        lat.close()
