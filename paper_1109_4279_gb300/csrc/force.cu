@@ -402,15 +402,19 @@ __global__ void __launch_bounds__(128) force_kernel(Geom g, const double2* __res
 int force_apply(qcd_ctx* c, const Rec& x, const Rec& y, double* F, cudaStream_t s) {
   if (x.prec != P64 || y.prec != P64) return QCD_ERR_ARG;
   QCD_TRY(ensure_gauge(c, P64, s));
-  // W (9 reals) and the four slots (32 reals) of a plane are 328 bytes per
-  // site: all six planes in one launch up to 4 GiB of them, else plane by plane
-  // (less memory than W alone used to take, and a large lattice fills the GPU
-  // with one plane)
+  // W (9 reals) and the four slots (32 reals) of a plane are 328 bytes per site: all
+  // six planes in one launch up to 4 GiB of them and where the device has room, else
+  // plane by plane (less memory than W alone used to take, the same sums in the same
+  // order, and a large lattice fills the GPU with one plane)
   const size_t per_plane = (size_t)c->V * 41 * sizeof(double);
-  const int group = 6 * per_plane <= ((size_t)4 << 30) ? 6 : 1;
+  int group = 6 * per_plane <= ((size_t)4 << 30) ? 6 : 1;
   const bool clover = c->p.csw != 0.0;
   Scratch mem;
-  if (clover) QCD_TRY(mem.get(c, kScratchForce, per_plane * group));
+  if (clover) {
+    int st = mem.get(c, kScratchForce, per_plane * group);
+    if (st == QCD_ERR_NOMEM && group > 1) st = mem.get(c, kScratchForce, per_plane * (group = 1));
+    QCD_TRY(st);
+  }
   double* W = (double*)mem.p;
   double* S = W + (size_t)c->V * 9 * group;
   const unsigned grid = (unsigned)((c->V + 127) / 128);

@@ -99,3 +99,24 @@ def test_all_contexts_keep_two_gib_at_most():
     assert torch.equal(outs[3], outs[0])
     for lat in lats[1:]:
         lat.close()
+
+
+def test_force_with_room_for_one_plane_only():
+    """All six planes' scratch is 1968 bytes per site, one plane's 328: the force then
+    goes plane by plane and adds the same numbers in the same order."""
+    from paper_1109_4279_gb300 import binding as B
+    dims, block = (8, 8, 8, 16), (4, 4, 4, 4)  # 16.1 MB, 2.7 MB; staged fields 3.1 MB
+    (a, c), rng = _lattices(2, dims, block, 63)
+    x, y = (torch.from_numpy(synth.gaussian_spinor(dims, rng)).cuda() for _ in range(2))
+    F, G = (torch.empty((a.V, 4, 8), dtype=torch.float64, device="cuda") for _ in range(2))
+    B.qcd_force(a.ctx, x, y, F)
+    a.close()  # (what it keeps counts towards the limit)
+    with _limit(c, 8_000_000):
+        B.qcd_force(c.ctx, x, y, G)
+    assert torch.equal(F, G)
+    with _limit(c, 8_000_000):
+        B.qcd_force(c.ctx, x, y, G)  # from the memory kept by the call before
+    B.qcd_force(c.ctx, y, x, F)
+    B.qcd_force(c.ctx, x, y, F)
+    assert torch.equal(F, G)
+    c.close()
