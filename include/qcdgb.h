@@ -343,12 +343,15 @@ int qcd_tune_block(const qcd_params* p, const double* U, const double* b, int is
  * 256 for DF64) and its threads per site `tps`: 1, or 2 for 16-bit storage
  * (QCD_PREC_F16 / BF16: two threads share a site, each taking two of the four
  * directions and half of the spin components, in CTAs of 256;
- * QCD_ERR_UNSUPPORTED otherwise).  qcd_get_launch reads the current shape.
+ * QCD_ERR_UNSUPPORTED otherwise).  While no size was set for FP64, a lattice whose
+ * sites alone do not fill the GPU takes a form that shares a site among four warps
+ * (CTAs of 128 threads); a size set here always applies.  qcd_get_launch reads the
+ * current shape.
  * qcd_set_sap_tile sets how many right-hand sides one CTA of a batched SAP
  * sweep solves with one staging of its block's fields (1..64; 0
  * restores the default: the largest tile that keeps four CTAs per SM);
  * qcd_get_sap_tile returns the tile a solve of nrhs right-hand sides uses.
- * Results do not depend on any of these.
+ * Results do not depend on any of these beyond rounding.
  */
 int qcd_set_launch(qcd_ctx* ctx, int prec, int threads, int tps);
 int qcd_get_launch(const qcd_ctx* ctx, int prec, int* threads, int* tps);

@@ -806,6 +806,7 @@ int qcd_set_launch(qcd_ctx* c, int prec, int threads, int tps) {
   ++c->gen;  // captured graphs hold the launch shape
   c->dirac_threads[prec] = threads;
   c->dirac_tps[prec] = tps;
+  if (prec == QCD_PREC_F64) c->f64_threads_set = true;
   return QCD_OK;
 }
 

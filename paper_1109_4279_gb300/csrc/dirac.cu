@@ -944,7 +944,8 @@ __global__ void __launch_bounds__(4 * kSplitSites, 4) dirac_split_kernel(Geom g,
   }
 }
 
-// The split form where its warps fill the SM quarters better: FP64 operations that
+// The split form where its warps fill the SM quarters better (and no CTA size was set
+// for the operator, which applies to the other form): FP64 operations that
 // one quarter runs through, per warp 1150 (one thread per site, right-hand sides in
 // turn) or 306 (split, right-hand sides side by side), times the warps it gets.
 // One right-hand side, one thread per site / split: 256 sites 41 / 15 us, 8192 43 / 25,
@@ -1028,7 +1029,7 @@ int dirac_apply(qcd_ctx* c, const Rec& in, const Rec& out, int dagger, cudaStrea
     QCD_LAUNCHED();
     return QCD_OK;
   }
-  if (prec == P64 && use_split(c, nrhs)) {
+  if (prec == P64 && !c->f64_threads_set && use_split(c, nrhs)) {
     const dim3 g2((unsigned)((c->V + kSplitSites - 1) / kSplitSites), nrhs);
     if (dagger)
       dirac_split_kernel<1, false><<<g2, 4 * kSplitSites, 0, s>>>(c->g, U, A, in.ptr(), out.ptr(), FieldPtr{}, mask,

@@ -190,6 +190,7 @@ struct qcd_ctx {
   // over the SMs and leave a smaller last wave (FP64 on 16^3 x 32 271 us with 64
   // threads, 305 with 256, on 8^4 43 and 79; 16-bit storage 15.2 and 16.9).
   int dirac_threads[5] = {64, 128, 128, 128, qcd::kDfThreads};
+  bool f64_threads_set = false;  // by qcd_set_launch: the FP64 operator is not split over warps then
   int sap_rt = 0;  // right-hand sides per CTA of batched SAP launches (0: sap_tile's default)
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)
   void* scratch[2] = {nullptr, nullptr};  // kept staging buffers (qcd::Scratch)
