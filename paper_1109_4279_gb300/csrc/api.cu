@@ -255,6 +255,7 @@ int qcd_create(qcd_ctx** out, const qcd_params* p) {
   int st = setup_geometry(c);
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int prec : {P64, P32, P16, PB16}) c->dirac_threads[prec] = dirac_cta(c->V, c->sms);
   if (st == QCD_OK) {
     if (dev_malloc(&c->d_scalars, 64 * 1024) != cudaSuccess || cudaMallocHost(&c->h_scalars, 64 * 1024) != cudaSuccess ||
         cudaMemset(c->d_scalars, 0, 64 * 1024) != cudaSuccess)

@@ -44,9 +44,23 @@ inline int chunks(int prec, int nreal) {
 // CTA size of the double-float kernels: their registers allow 8 warps per SM, and
 // two CTAs of four fill an SM's gaps better than one of eight
 static constexpr int kDfThreads = 128;
-// and of the FP64 ones: a warp's operation holds a quarter of an SM's FP64 unit for
-// 64 cycles, so a small lattice's warps have to be spread over the quarters
+// and of the FP64 residual and even/odd kernels: a warp's operation holds a quarter of
+// an SM's FP64 unit for 64 cycles, so a small lattice's warps have to be spread over
+// the quarters
 static constexpr int kF64Threads = 64;
+
+// Default CTA size of the other operators.  Small CTAs spread a small lattice over the
+// SMs and leave a smaller last wave (16-bit storage on 16^3 x 32 14.5 us with 128
+// threads, 16.6 with 256; FP64 on 8^4 43 and 78, on 16^3 x 32 271 and 304, and the same
+// with 64 as with 128).  Where the lattice runs in one wave and the busiest SM gets as
+// many threads either way, CTAs of 256 keep more of a block's neighbours on one SM: 12
+// FP16 right-hand sides on 16^4 78 us with 256 threads, 82 with 128, 12 FP32 ones on
+// 16 x 12^3 47 and 49; FP64 on 73728 sites 156 and 158.
+inline int dirac_cta(long long V, int sms) {
+  const long long n128 = (V + 127) / 128, n256 = (V + 255) / 256;
+  const long long busiest128 = (n128 + sms - 1) / sms * 128, busiest256 = (n256 + sms - 1) / sms * 256;
+  return busiest128 <= 512 && busiest256 <= busiest128 ? 256 : 128;
+}
 
 // doubles at the start of every right-hand side's partial sums; the first word is
 // the count of finished CTAs, 0 between kernels
@@ -185,11 +199,9 @@ struct qcd_ctx {
   bool prof = false;
   qcd::Timer timers[QCD_KERNEL_COUNT];
   std::vector<cudaEvent_t> event_pool;
-  // launch shape chosen by the autotuner
-  // CTA size of the operator kernel per precision.  Small CTAs spread a small lattice
-  // over the SMs and leave a smaller last wave (FP64 on 16^3 x 32 271 us with 64
-  // threads, 305 with 256, on 8^4 43 and 79; 16-bit storage 15.2 and 16.9).
-  int dirac_threads[5] = {64, 128, 128, 128, qcd::kDfThreads};
+  // launch shape: the default of qcd::dirac_cta (set by qcd_create), what
+  // qcd_autotune chose, or what qcd_set_launch set
+  int dirac_threads[5] = {128, 128, 128, 128, qcd::kDfThreads};  // CTA size of the operator kernel per precision
   bool f64_threads_set = false;  // by qcd_set_launch: the FP64 operator is not split over warps then
   int sap_rt = 0;  // right-hand sides per CTA of batched SAP launches (0: sap_tile's default)
   int dirac_tps[5] = {1, 1, 1, 1, 1};  // threads per site of the operator kernel (2: 16-bit storage only)

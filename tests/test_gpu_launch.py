@@ -32,3 +32,21 @@ def test_fp64_size_that_was_set(orc, dims, block):
     assert all(torch.equal(o, outs[0]) for o in outs)
     for o in (default[0], outs[0]):
         assert abs(o.cpu().numpy() - ref).max() < 1e-13 * abs(ref).max()
+
+
+def test_default_size(orc):
+    """The default CTA size at the lattice sizes around which it changes (an SM's CTAs of
+    128 and of 256 threads hold as many threads at the most from 19457 to 38912 and from
+    58369 to 77824 sites on 152 SMs), and the operator with it."""
+    import numpy as np
+    from paper_1109_4279_gb300 import binding as B
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for dims, block in (((4, 4, 4, 4), (2, 2, 2, 2)), ((8, 8, 16, 16), (4, 4, 4, 4)), ((16, 12, 12, 12), (4, 6, 2, 2)),
+                        ((8, 16, 16, 16), (4, 4, 4, 4)), ((24, 12, 12, 12), (4, 6, 2, 2)), ((16, 16, 16, 16), (4, 4, 4, 4)),
+                        ((16, 16, 16, 20), (4, 4, 4, 2)), ((32, 16, 16, 16), (4, 4, 4, 4))):
+        V = int(np.prod(dims))
+        per_sm = [-(-(-(-V // t)) // sms) * t for t in (128, 256)]
+        want = 256 if per_sm[1] <= per_sm[0] <= 512 else 128
+        lat = B.Lattice(dims, block, 0.1, 1.3)
+        assert [B.qcd_get_launch(lat.ctx, p) for p in ("f64", "f32", "f16", "bf16", "df64")] == [(want, 1)] * 4 + [(128, 1)]
+        lat.close()
