@@ -20,6 +20,11 @@
 
 namespace qcd {
 
+// part of the key: entries that were timed with other kernels are not applied (1, without
+// a mark: before the operator's defaults depended on the lattice and its FP64 form on
+// the number of right-hand sides)
+static constexpr int kTuneVersion = 2;
+
 static std::string tune_key(qcd_ctx* c, int nrhs) {
   cudaDeviceProp prop;
   int dev = 0;
@@ -30,7 +35,8 @@ static std::string tune_key(qcd_ctx* c, int nrhs) {
     if (ch == '"' || ch == '\\') ch = '_';
   std::ostringstream k;
   k << name << "|" << c->p.dims[0] << "x" << c->p.dims[1] << "x" << c->p.dims[2] << "x" << c->p.dims[3] << "|b"
-    << c->p.block[0] << "x" << c->p.block[1] << "x" << c->p.block[2] << "x" << c->p.block[3] << "|nrhs" << nrhs;
+    << c->p.block[0] << "x" << c->p.block[1] << "x" << c->p.block[2] << "x" << c->p.block[3] << "|nrhs" << nrhs << "|v"
+    << kTuneVersion;
   return k.str();
 }
 
@@ -93,6 +99,7 @@ static void cache_store(const char* path, const std::string& key, const int v[kT
 
 static void tune_apply(qcd_ctx* c, const int v[kTuneFields]) {
   for (int p = 0; p < 5; ++p) c->dirac_threads[p] = v[p];
+  c->f64_threads_set = false;
   c->dirac_tps[P64] = c->dirac_tps[P32] = c->dirac_tps[PDF] = 1;
   c->dirac_tps[P16] = v[5];
   c->dirac_tps[PB16] = v[6];
@@ -125,7 +132,8 @@ extern "C" int qcd_autotune(qcd_ctx* c, int nrhs, const char* cache_path) {
   if (!c || nrhs < 1) return QCD_ERR_ARG;
   if (!c->clover_built) return QCD_ERR_STATE;
   const std::string key = tune_key(c, nrhs);
-  int best[kTuneFields] = {256, 256, 256, 256, 256, 1, 1, 0};
+  const int cta = dirac_cta(c->V, c->sms);
+  int best[kTuneFields] = {cta, cta, cta, cta, kDfThreads, 1, 1, 0};  // the defaults
   ++c->gen;  // the operator's launch shape changes under captured graphs
   if (cache_lookup(cache_path, key, best)) {
     tune_apply(c, best);
@@ -137,9 +145,15 @@ extern "C" int qcd_autotune(qcd_ctx* c, int nrhs, const char* cache_path) {
   c->prof = false;
   int st = QCD_OK;
   // operator: CTA size with one thread per site, for 16-bit storage also the
-  // two-threads-per-site form
+  // two-threads-per-site form.  Where the FP64 operator shares a site among four warps
+  // there is no size to choose.
+  c->f64_threads_set = false;
   const int cand[4][2] = {{128, 1}, {256, 1}, {512, 1}, {256, 2}};
   for (int p = P64; p <= PDF && st == QCD_OK; ++p) {
+    if (p == P64 && use_split(c, nrhs)) {
+      c->dirac_threads[p] = best[p];
+      continue;
+    }
     Rec a, b;
     st = rec_alloc(a, p, 24, c->V * nrhs);
     if (st == QCD_OK) st = rec_alloc(b, p, 24, c->V * nrhs);

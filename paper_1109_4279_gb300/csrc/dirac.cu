@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(4 * kSplitSites, 4) dirac_split_kernel(Geom g,
 // turn) or 306 (split, right-hand sides side by side), times the warps it gets.
 // One right-hand side, one thread per site / split: 256 sites 41 / 15 us, 8192 43 / 25,
 // 16384 43 / 45, 32768 80 / 74, 41472 107 / 94, 65536 147 / 146, 131072 271 / 275.
-static bool use_split(const qcd_ctx* c, int nrhs) {
+bool use_split(const qcd_ctx* c, int nrhs) {
   if (nrhs > 65535) return false;  // (a grid dimension)
   const long long q = 4LL * c->sms;
   const long long whole = (c->V + 32 * q - 1) / (32 * q) * nrhs, split = (c->V * nrhs + 8 * q - 1) / (8 * q);

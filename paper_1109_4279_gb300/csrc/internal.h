@@ -304,6 +304,8 @@ int build_clover(qcd_ctx* c, cudaStream_t s);
 int ensure_clover(qcd_ctx* c, int prec, cudaStream_t s);
 
 // ---- dirac.cu
+// whether the FP64 operator shares a site among four warps (unless a CTA size was set)
+bool use_split(const qcd_ctx* c, int nrhs);
 // out = D in (dagger: D^+); fields in one precision
 // nrhs > 1: in/out hold nrhs fields back to back (V sites apart)
 // mask (device, nrhs flags, may be null): right-hand sides whose flag is 0 are skipped
