@@ -592,8 +592,7 @@ __device__ __forceinline__ Spinor<T> hops_pair(const ST& st, int n, int r, const
 }
 
 // Pair exchange through shared memory: xb holds [2][12][np] reals (np = site
-// pairs per half, a multiple of 32).  Both calls below contain a barrier and
-// must be reached by every thread of the CTA.
+// pairs per half, a multiple of 32).
 
 // barrier of the two warps that hold pairs 32 w .. 32 w + 31 (warp w of each
 // half): named barrier 1 + w (np / 32 <= 8 of them; barrier 0 is the CTA-wide one)
@@ -969,7 +968,8 @@ __host__ __device__ __forceinline__ int pairs_per_half(int Vbh) { return (Vbh + 
 // them); otherwise exactly one, right-hand side 0, and the loop folds away
 // Threads: the largest block whose fields fit in shared memory has 512 sites in
 // 16-bit form, 320 in FP32 and 144 in FP64 -- two threads per pair of sites, in
-// whole warps per half -- so the wider arithmetic gets more registers.
+// whole warps per half -- so the wider arithmetic gets more registers (set_smem_attr
+// refuses a block that needs more threads).
 template <int P>
 struct SapThreads {
   static constexpr int most = P == P64 ? 192 : (P == P32 ? 320 : 512);
@@ -1281,7 +1281,7 @@ __global__ void __launch_bounds__(SapThreads<P>::most) sap_sweep_kernel(SapArgs 
       }
     }
 
-    // ---- outputs: solution, block residual (r on even, 0 on odd), faces
+    // ---- outputs: solution, block residual (r; on even sites only, see above), faces
     constexpr int PS = PsiPrec<P>::value;
     typedef typename std::conditional<PS == P64, double, float>::type TS;
     // what the partner needs: chi_o goes to t and chi_e to r (both read for the last
@@ -1368,7 +1368,7 @@ static int set_smem_attr_vb(size_t smem) {
 template <int P, typename T>
 static int set_smem_attr(const Geom& g, int maxsm) {
   const size_t smem = sap_smem_bytes<P, T>(g);
-  if (smem > (size_t)maxsm) return QCD_ERR_UNSUPPORTED;
+  if (smem > (size_t)maxsm || 2 * pairs_per_half(g.Vbh) > SapThreads<P>::most) return QCD_ERR_UNSUPPORTED;
   if constexpr (P == P16 || P == PB16) {
     if (sap_vb_key(g.Vb) == 256) return set_smem_attr_vb<P, T, 256>(smem);
     if (sap_vb_key(g.Vb) == 512) return set_smem_attr_vb<P, T, 512>(smem);
