@@ -6,8 +6,11 @@
  * host or device pointers as stated; sizes are element counts; no C++ or torch
  * types cross this boundary.  Every function returns an int status: QCD_OK (0)
  * or a negative QCD_ERR_* code (see qcd_status_string); no exception and no
- * exit() ever crosses the ABI.  A context is not thread-safe; separate contexts
- * are independent.
+ * exit() ever crosses the ABI.  Separate contexts are independent.  One context
+ * is used by one thread at a time, except that several threads may call
+ * qcd_apply_D and qcd_force on it at once, each on a stream of its own, while
+ * profiling is off and after a first qcd_apply_D in each precision they use (it
+ * makes that precision's copies of the links and the clover term).
  *
  * Method: "Solving the Dirac equation on QPACE" (A. Nobile, Lattice 2010,
  * arXiv:1109.4279).  The solver inverts the Wilson-Dirac operator with clover

@@ -109,3 +109,42 @@ def test_first_solve_while_another_thread_captures_a_blocking_stream():
     assert torch.equal(xs[1], xs[0]) and torch.equal(xs[2], xs[0])
     for lat in contexts:
         lat.close()
+
+
+def test_force_and_operator_of_one_context_from_several_threads():
+    """qcd_apply_D and qcd_force of one context at once, each thread on its own stream:
+    the staging memory of a call is its own until it returns (bit for bit)."""
+    from paper_1109_4279_gb300 import binding as B
+    dims, block, n = (8, 8, 8, 8), (4, 4, 4, 4), 4
+    U, rng = synth.gauge_field(dims, 0.5, 55)
+    lat = B.Lattice(dims, block, 0.1, 1.3)
+    lat.load_gauge(torch.from_numpy(U).cuda())
+    psi = torch.from_numpy(synth.gaussian_spinor(dims, rng, nrhs=n + 1)).cuda()
+    D = [torch.empty_like(psi[0]) for _ in range(n)]
+    F = [torch.empty((lat.V, 4, 8), dtype=torch.float64, device="cuda") for _ in range(n)]
+    for k in range(n):
+        B.qcd_apply_D(lat.ctx, psi[k], D[k], prec="f32")
+        B.qcd_force(lat.ctx, psi[k], psi[k + 1], F[k])
+    got = [[(torch.empty_like(D[k]), torch.empty_like(F[k])) for _ in range(8)] for k in range(n)]
+    streams = [torch.cuda.Stream() for _ in range(n)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            with torch.cuda.stream(streams[k]):
+                for d, f in got[k]:
+                    B.qcd_apply_D(lat.ctx, psi[k], d, prec="f32")
+                    B.qcd_force(lat.ctx, psi[k], psi[k + 1], f)
+        except Exception as e:  # (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(n)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    assert all(torch.equal(d, D[k]) and torch.equal(f, F[k]) for k in range(n) for d, f in got[k])
+    lat.close()
