@@ -55,7 +55,7 @@ DW_FLOPS = 1824.0  # 1320 hopping + 504 clover per site
 # dram__bytes_write.sum, 24^3x48 lattice, 331,776 solved sites per launch); valid
 # for the kernel sources whose hash is stored with it and that block shape,
 # scaled by solved sites
-SAP_TRAFFIC = {"bytes_per_site": 542.7, "src_sha": "76abbcdd1ea84a0e", "block": (8, 4, 4, 4)}
+SAP_TRAFFIC = {"bytes_per_site": 542.7, "src_sha": "534028a9f0f2077b", "block": (8, 4, 4, 4)}
 
 
 def sap_src_sha():
