@@ -317,7 +317,9 @@ int qcd_hmc_trajectory(qcd_ctx* ctx, double* U, double* pi, const double* eta, d
  * nrhs: right-hand sides per call the tuning should reflect (the operator
  * timing applies that many operators back to back).  cache_path (may be
  * NULL): a JSON file read before tuning (a matching entry is applied without
- * timing) and rewritten after it, keyed by GPU name, dims, block and nrhs.
+ * timing) and rewritten after it, keyed by GPU name, dims, block, nrhs and a
+ * version of the kernels; entries under other keys are left in it.  The FP64 size
+ * is not timed where a site is shared among four warps (see qcd_set_launch).
  * Needs qcd_load_gauge and qcd_build_clover first.
  */
 int qcd_autotune(qcd_ctx* ctx, int nrhs, const char* cache_path);
